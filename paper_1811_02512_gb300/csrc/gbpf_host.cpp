@@ -523,6 +523,49 @@ pf_status build_tail(pf_ctx *ctx, HostMat &H, MakePieces &make_pieces, RunEnds &
 
 // Device layout of one analysed matrix in level order (see DevMat).
 pf_status build_layout(pf_ctx *ctx, HostMat &H) {
+// Where the block factor changes from a warp per column to a warp per target
+// (see DevMat): the level above which the level-by-level form is the faster
+// one by the estimates below, in microseconds as measured on GB300.  By
+// columns a level costs its heaviest column (about 3, and 0.03 per update
+// term: the terms of a column run on one warp) per round of columns; by
+// targets a barrier and one pass of 32 terms per lane group and round of
+// targets (about 1, 1.5 and 0.6).  On a 20,000-bus grid the columns of the
+// narrow top carry thousands of terms each, all on one warp: the Newton
+// launch of four steps took 114 ms with a warp per column throughout.
+void split_block_factor(HostMat &H) {
+    H.jlt.assign(H.nlev + 1, 0);
+    for (int l = 0; l <= H.nlev; l++) H.jlt[l] = H.Cp[H.lvl_ptr[l]] + H.lvl_ptr[l];
+    const int warps[2] = {kSweepWarps, kSweepWarps * kClCtas};
+    for (int w = 0; w < 2; w++) {
+        H.jl0[w] = H.nlev;
+        double gain = 0.0, best = 0.0;
+        for (int l = H.nlev - 1; l >= 0; l--) {
+            int heavy = 0, longest = 0;
+            for (int c = H.lvl_ptr[l]; c < H.lvl_ptr[l + 1]; c++) {
+                const int t0 = H.Cp[c] + c, t1 = H.Cp[c + 1] + c + 1;
+                heavy = std::max(heavy, H.gp[t1] - H.gp[t0]);
+                for (int t = t0; t < t1; t++) longest = std::max(longest, H.gp[t + 1] - H.gp[t]);
+            }
+            auto rounds = [](int n, int by) { return double((n + by - 1) / by); };
+            const double by_col = rounds(H.lvl_ptr[l + 1] - H.lvl_ptr[l], warps[w]) * (3.0 + 0.03 * heavy);
+            const double by_tgt = 1.0 + rounds(H.jlt[l + 1] - H.jlt[l], warps[w]) * (1.5 + 0.6 * rounds(longest, 32));
+            gain += by_col - by_tgt;
+            if (gain > best) {
+                best = gain;
+                H.jl0[w] = l;
+            }
+        }
+        H.jct[w] = H.lvl_ptr[H.jl0[w]];
+    }
+    const int c0 = std::min(H.jct[0], H.jct[1]);
+    H.jg0 = H.Cp[c0] + c0;
+    H.jtcol.clear();
+    for (int c = c0; c < H.n; c++) {
+        H.jtcol.push_back(~c);
+        H.jtcol.insert(H.jtcol.end(), size_t(H.Cp[c + 1] - H.Cp[c]), c);
+    }
+}
+
     const int n = H.n;
     const int64_t nnz = H.Lp[n];
     // level order: steps sorted by (level, step)
@@ -777,6 +820,7 @@ pf_status build_layout(pf_ctx *ctx, HostMat &H) {
     for (int c = 0; c < n; c++)
         for (int p = H.Cp[c]; p < H.Cp[c + 1]; p++) H.srcT[p] = ypos(ctx, H.bus_new[c], H.bus_new[H.Cr[p]]);
     H.jD = 0;
+    split_block_factor(H);
     H.jDi = pad32(4 * int64_t(n));
     H.jLc = H.jDi + pad32(4 * int64_t(n));
     H.jUc = H.jLc + pad32(4 * nnz);
@@ -1371,6 +1415,13 @@ pf_status upload_matrix(pf_ctx *ctx, const HostMat &H, DevMat &D) {
     TRY(upload(ctx, &D.pbJ, H.pbJ.data(), H.pbJ.size()));
     TRY(upload_padded(ctx, &D.srcT, H.srcT));
     D.npfJ = int(H.pfJ.size());
+    TRY(upload_padded(ctx, &D.jlt, H.jlt));
+    TRY(upload_padded(ctx, &D.jtcol, H.jtcol));
+    D.jg0 = H.jg0;
+    for (int w = 0; w < 2; w++) {
+        D.jl0[w] = H.jl0[w];
+        D.jct[w] = H.jct[w];
+    }
     D.npbJ = int(H.pbJ.size());
     D.jD = H.jD; D.jDi = H.jDi; D.jLc = H.jLc; D.jUc = H.jUc; D.jLr = H.jLr; D.jUr = H.jUr;
     D.jstride = H.jstride;

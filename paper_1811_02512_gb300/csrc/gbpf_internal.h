@@ -141,6 +141,13 @@ struct DevMat {
     int npfJ = 0, npbJ = 0;
     Piece *pfJ = nullptr, *pbJ = nullptr;
     int *srcT = nullptr;       // [nnz] Ybus position of the transposed entry (c, r) of each slot
+    // Top levels of the block factor, factorised level by level with a warp
+    // per target: from level jl0[w] (first column jct[w]) up, w = 0 for the
+    // warps of one block per case, 1 for a cluster's.  jlt[l]: first target
+    // (Cp[c] + c of the level's first column) of level l, [nlev + 1]; jtcol:
+    // column c of every target from jg0 on, ~c for a diagonal.
+    int jl0[2] = {0, 0}, jct[2] = {0, 0}, jg0 = 0;
+    int *jlt = nullptr, *jtcol = nullptr;
     int jD = 0, jDi = 0, jLc = 0, jUc = 0, jLr = 0, jUr = 0, jstride = 0;  // block layout (elements)
 };
 
@@ -260,6 +267,8 @@ struct HostMat {
     std::vector<int> Ap, Aj, Apos;    // off-diagonal pattern of A by row (both triangles, no fill)
     std::vector<Piece> pfJ, pbJ;
     std::vector<int> srcT;
+    int jl0[2] = {0, 0}, jct[2] = {0, 0}, jg0 = 0;
+    std::vector<int> jlt, jtcol;
     int jD = 0, jDi = 0, jLc = 0, jUc = 0, jLr = 0, jUr = 0, jstride = 0;
     std::vector<Piece> pf, pb;
     int offDi = 0, offLc = 0, offLr = 0, stride = 0;

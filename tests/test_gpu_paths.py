@@ -1,0 +1,46 @@
+"""GPU checks of the size-dependent code paths at the sizes where they change,
+against the CPU oracle."""
+import numpy as np
+import pytest
+
+from paper_1811_02512_gb300 import gbpf, gridgen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _loaded(raw, lam=1.0 / 32):
+    return raw.scaled_network(lam)
+
+
+# ncase 1: a 16-block cluster per case; ncase 20: one block per case.  n = 3
+# and 30 put every level in the top part of the block factor or nearly so.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("ncase", [1, 20])
+@pytest.mark.parametrize("n", [3, 30, 700])
+def test_newton_factor_top_and_adjoint(oracle, n, ncase, prec):
+    raw = gridgen.small_raw(n, 11) if n < 100 else gridgen.delaunay_raw(n, 11)
+    case = _loaded(raw)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    g = gbpf.Grid(case)
+    g.set_cases(ncase)
+    vm = torch.zeros((ncase, n), dtype=torch.float64, device="cuda")
+    va = torch.zeros_like(vm)
+    st, res = gbpf.pf_run_to_tol(g.ctx, gbpf.run_opts(gbpf.PF_NR, p, tol=1e-11, max_iter=30), vm, va, ncase)
+    assert st == gbpf.PF_OK
+    J = torch.empty(ncase, dtype=torch.float64, device="cuda")
+    gva, gvm, dP, dQ = (torch.empty_like(vm) for _ in range(4))
+    gbpf.pf_objective(g.ctx, vm, va, J, gva, gvm)
+    gbpf.pf_adjoint(g.ctx, p, vm, va, gva, gvm, dP, dQ, ncase)
+    rc, vm0, va0, _, _ = oracle.power_flow(case, oracle.NR, tol=1e-12)
+    assert rc == oracle.OK
+    aP, aQ, _ = oracle.adjoint(case, vm0, va0)
+    scale = max(np.abs(aP).max(), np.abs(aQ).max())
+    # a mismatch of 1e-11 defines the state to the inverse Jacobian's norm
+    # times that (the adjoint of a per-bus sum bounds it: below 1e3 here)
+    for c in (0, ncase - 1):
+        assert np.abs(vm[c].cpu().numpy() - vm0).max() <= 1e-8
+        assert np.abs(va[c].cpu().numpy() - va0).max() <= 1e-8
+        assert np.abs(dP[c].cpu().numpy() - aP).max() <= 1e-7 * scale
+        assert np.abs(dQ[c].cpu().numpy() - aQ).max() <= 1e-7 * scale
+    g.close()
