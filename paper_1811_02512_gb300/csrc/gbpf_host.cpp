@@ -521,8 +521,6 @@ pf_status build_tail(pf_ctx *ctx, HostMat &H, MakePieces &make_pieces, RunEnds &
     return PF_OK;
 }
 
-// Device layout of one analysed matrix in level order (see DevMat).
-pf_status build_layout(pf_ctx *ctx, HostMat &H) {
 // Where the block factor changes from a warp per column to a warp per target
 // (see DevMat): the level above which the level-by-level form is the faster
 // one by the estimates below, in microseconds as measured on GB300.  By
@@ -566,6 +564,8 @@ void split_block_factor(HostMat &H) {
     }
 }
 
+// Device layout of one analysed matrix in level order (see DevMat).
+pf_status build_layout(pf_ctx *ctx, HostMat &H) {
     const int n = H.n;
     const int64_t nnz = H.Lp[n];
     // level order: steps sorted by (level, step)
@@ -819,8 +819,8 @@ void split_block_factor(HostMat &H) {
     H.srcT.assign(nnz, -1);
     for (int c = 0; c < n; c++)
         for (int p = H.Cp[c]; p < H.Cp[c + 1]; p++) H.srcT[p] = ypos(ctx, H.bus_new[c], H.bus_new[H.Cr[p]]);
-    H.jD = 0;
     split_block_factor(H);
+    H.jD = 0;
     H.jDi = pad32(4 * int64_t(n));
     H.jLc = H.jDi + pad32(4 * int64_t(n));
     H.jUc = H.jLc + pad32(4 * nnz);
