@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdint>
 
+#include "gbpf_fx.cuh"
 #include "gbpf_internal.h"
 
 namespace gbpf {
@@ -860,6 +861,205 @@ __device__ __forceinline__ void bus_injection(const DevNet &dn, int i, int outag
     bus_current(dn, i, outage, e, f, ir, ii);
     P = e[i] * ir + f[i] * ii;
     Q = f[i] * ir - e[i] * ii;
+}
+
+// ------------------------------------------------------------ fixed point
+
+constexpr int kFxNone = int(0x80000000u);
+
+// The current at bus i in units 2^-(ysc[i] + 1), from the fixed-point
+// admittance row and the voltages ef[k * st] = {e h, e l, f h, f l} (units
+// 2^-58, |V| < 2); the outaged branch's terms are taken out as in
+// bus_current.  Twelve integer multiply-adds an entry, where the FP64 form
+// has four multiply-adds of 64 cycles: the nodal mismatch of the 10,000-bus
+// batch was bound by those.  CHECK: returns false when a voltage is kFxNone
+// (the outaged branch's other end is a neighbour too).
+template <bool CHECK>
+__device__ __forceinline__ bool fx_bus_current(const DevNet &dn, int i, int outage, const int4 *ef, int st,
+                                               long long &ir_out, long long &ii_out) {
+    FxAcc ir{0, 0}, ii{0, 0};
+    bool ok = !CHECK || dn.ysc[i] != kFxNoScale;
+    auto term = [&](const int4 &y, const int4 &v) {
+        fx_mac(ir, y.x, y.y, v.x, v.y);
+        fx_mac(ir, -y.z, -y.w, v.z, v.w);
+        fx_mac(ii, y.x, y.y, v.z, v.w);
+        fx_mac(ii, y.z, y.w, v.x, v.y);
+    };
+    // four entries at a time, all loads first; the cross terms of four
+    // entries stay below 2^62 and are carried before the next four
+    const int pe = dn.rowptr[i + 1];
+    for (int p = dn.rowptr[i]; p < pe; p += 4) {
+        int k[4];
+        int4 y[4], v[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            k[u] = p + u < pe ? dn.col[p + u] : i;
+            y[u] = p + u < pe ? dn.Yx[p + u] : make_int4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) v[u] = ef[(long long)k[u] * st];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (CHECK) ok &= v[u].x != kFxNone;
+            if (p + u < pe) term(y[u], v[u]);
+        }
+        if (p + 4 < pe) {
+            fx_carry(ir);
+            fx_carry(ii);
+        }
+    }
+    if (outage >= 0 && dn.bstatus[outage] && (i == dn.bf[outage] || i == dn.bt[outage])) {
+        const bool from = i == dn.bf[outage];
+        const int o = from ? dn.bt[outage] : dn.bf[outage], q = dn.ysc[i];
+        const double *t = dn.bry + 8LL * outage;
+        const FxLimbs gs = fx_split(-fx_from_double(t[from ? 0 : 2], q)), bs = fx_split(-fx_from_double(t[from ? 1 : 3], q));
+        const FxLimbs gm = fx_split(-fx_from_double(t[4], q)), bm = fx_split(-fx_from_double(t[5], q));
+        fx_carry(ir);
+        fx_carry(ii);
+        term(make_int4(gs.h, gs.l, bs.h, bs.l), ef[(long long)i * st]);
+        term(make_int4(gm.h, gm.l, bm.h, bm.l), ef[(long long)o * st]);
+    }
+    ir_out = fx_sum<3>(ir);
+    ii_out = fx_sum<3>(ii);
+    return ok;
+}
+
+// P = e ir + f ii (Q = f ir - e ii) in units 2^-(ysc + 2).
+__device__ __forceinline__ long long fx_power(bool q, const int4 &v, long long ir, long long ii) {
+    const FxLimbs r = fx_split(ir), m = fx_split(ii);
+    FxAcc s{0, 0};
+    if (!q) {
+        fx_mac(s, v.x, v.y, r.h, r.l);
+        fx_mac(s, v.z, v.w, m.h, m.l);
+    } else {
+        fx_mac(s, v.z, v.w, r.h, r.l);
+        fx_mac(s, -v.x, -v.y, m.h, m.l);
+    }
+    return fx_sum<3>(s);
+}
+
+// a / V as a double: a in units 2^-q, iv = 1 / V in units 2^-60.
+__device__ __forceinline__ double fx_over_v(long long a, int q, long long iv) {
+    const bool neg = (a < 0) != (iv < 0);
+    const unsigned long long m = a < 0 ? 0ull - static_cast<unsigned long long>(a) : static_cast<unsigned long long>(a);
+    if (m == 0ull) return 0.0;
+    const int lz = fx_clz(m);
+    const unsigned long long w = static_cast<unsigned long long>(iv < 0 ? -iv : iv) << 2;
+    const long long u = static_cast<long long>(fx_umulhi(m << lz, w) >> 1);  // a 2^(lz + q) iv 2^-1
+    return fx_to_double(neg ? -u : u, lz + q - 3);
+}
+
+__device__ __forceinline__ int4 fx_pack(long long e, long long f) {
+    const FxLimbs a = fx_split(e), b = fx_split(f);
+    return make_int4(a.h, a.l, b.h, b.l);
+}
+
+// e + jf of (V, theta) within the ranges of fx_state_ok.
+__device__ __forceinline__ int4 fx_polar(double vm, double va) {
+    long long s, c;
+    fx_sincos(va, s, c);
+    const long long v = fx_from_double(vm, kFxV);
+    return fx_pack(fx_scale_v(v, c), fx_scale_v(v, s));
+}
+
+// The same from V and theta in units 2^-60.
+__device__ __forceinline__ int4 fx_polar60(long long vv, long long th) {
+    long long s, c;
+    fx_sincos60(th, s, c);
+    const long long v = (vv + 2) >> 2;
+    return fx_pack(fx_scale_v(v, c), fx_scale_v(v, s));
+}
+// fx_vm_ok for V in units 2^-60.
+__device__ __forceinline__ bool fx_v60_ok(long long vv) {
+    const long long v = vv < 0 ? -vv : vv;
+    return v >= (9ll << 56) && v < (31ll << 56);
+}
+
+// 9/16 <= |V| < kFxVmax, |theta| < kFxThMax (integer compares; NaN fails).
+__device__ __forceinline__ bool fx_vm_ok(double v) {
+    const unsigned h = unsigned(__double2hiint(v)) & 0x7fffffffu;
+    return h - 0x3fe20000u < 0x3fff0000u - 0x3fe20000u;
+}
+__device__ __forceinline__ bool fx_va_ok(double t) {
+    return (unsigned(__double2hiint(t)) & 0x7fffffffu) < 0x401f0000u;
+}
+
+// e + jf rotated by d (units 2^-60, |d| <= 0.2); every lane of the warp that
+// is here takes the short series when all can.
+__device__ __forceinline__ int4 fx_rotate(const int4 &v, long long d) {
+    long long sd, cm;
+    const bool small = (d < 0 ? -d : d) < (1ll << 50);
+    fx_small_sincos(d, __all_sync(__activemask(), small), sd, cm);
+    const FxLimbs s = fx_split(sd), c = fx_split(cm);
+    FxAcc a{0, 0}, b{0, 0};
+    fx_mac(a, v.x, v.y, c.h, c.l);
+    fx_mac(a, v.z, v.w, s.h, s.l);
+    fx_mac(b, v.z, v.w, c.h, c.l);
+    fx_mac(b, -v.x, -v.y, s.h, s.l);
+    return fx_pack(fx_join(v.x, v.y) - fx_sum<0>(a), fx_join(v.z, v.w) - fx_sum<0>(b));
+}
+
+// e + jf scaled by 1 + r (r in units 2^-60, |r| < 1).
+__device__ __forceinline__ int4 fx_stretch(const int4 &v, long long r) {
+    const FxLimbs x = fx_split(r);
+    FxAcc a{0, 0}, b{0, 0};
+    fx_mac(a, v.x, v.y, x.h, x.l);
+    fx_mac(b, v.z, v.w, x.h, x.l);
+    return fx_pack(fx_join(v.x, v.y) + fx_sum<0>(a), fx_join(v.z, v.w) + fx_sum<0>(b));
+}
+
+// a b with both in units 2^-60, below 2 in magnitude.
+__device__ __forceinline__ long long fx_mul60(long long a, long long b) {
+    const FxLimbs x = fx_split(a), y = fx_split(b);
+    FxAcc s{0, 0};
+    fx_mac(s, x.h, x.l, y.h, y.l);
+    return fx_sum<0>(s);
+}
+
+// Bus states given by a caller may be out of the fixed-point range: their
+// entry is kFxNone, and what needs it takes the FP64 form.  An angle beyond
+// fx_sincos's range only goes through CUDA's sincos.
+__device__ __forceinline__ int4 fx_polar_any(double vm, double va) {
+    const unsigned h = unsigned(__double2hiint(vm)) & 0x7fffffffu, t = unsigned(__double2hiint(va)) & 0x7fffffffu;
+    if (h >= 0x3fff0000u || t >= 0x7ff00000u) return make_int4(kFxNone, 0, 0, 0);
+    if (t < 0x401f0000u) return fx_polar(vm, va);
+    double s, c;
+    sincos(va, &s, &c);
+    const long long v = fx_from_double(vm, kFxV);
+    return fx_pack(fx_scale_v(v, fx_from_double(c, 60)), fx_scale_v(v, fx_from_double(s, 60)));
+}
+
+// Angle step d of a bus in fixed point: e + jf rotated (or formed again from
+// V and the new angle va for a step beyond the series).  Returns whether the
+// bus left the fixed-point range (a NaN step does).
+__device__ __forceinline__ bool fx_angle_step(int4 *ef, double d, double vm, double va) {
+    const unsigned h = unsigned(__double2hiint(d)) & 0x7fffffffu;
+    if (h < 0x3fc99999u) {  // |d| < 0.2
+        *ef = fx_rotate(*ef, fx_from_double(d, 60));
+        return !fx_va_ok(va);
+    }
+    if (!fx_va_ok(va)) return true;
+    *ef = fx_polar(vm, va);
+    return false;
+}
+
+// Magnitude step d of a bus, vm the new magnitude: e + jf scaled by 1 + d/V
+// (formed again from the state for a large step) and the new 1/V.
+__device__ __forceinline__ bool fx_magnitude_step(int4 *ef, long long *iv, double d, double vm, double va) {
+    if (!fx_vm_ok(vm)) return true;
+    if ((unsigned(__double2hiint(d)) & 0x7fffffffu) < 0x3fd00000u)  // |d| < 1/4
+        *ef = fx_stretch(*ef, fx_mul60(fx_from_double(d, 60), *iv));
+    else
+        *ef = fx_polar(vm, va);
+    *iv = fx_recip(fx_from_double(vm, kFxV));
+    return false;
+}
+
+// State of one bus in fixed point: whether bus i of a case can start there
+// (V, theta and the specified injections in range).
+__device__ __forceinline__ bool fx_state_ok(const DevNet &dn, int i, double vm, double va, double psp, double qsp) {
+    const int q = dn.ysc[i] + 2;
+    return fx_vm_ok(vm) && fx_va_ok(va) && fx_fits(psp, q) && fx_fits(qsp, q);
 }
 
 }  // namespace

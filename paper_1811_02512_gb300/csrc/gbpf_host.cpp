@@ -24,6 +24,7 @@
 #include <set>
 #include <utility>
 
+#include "gbpf_fx.cuh"
 #include "gbpf_internal.h"
 
 using namespace gbpf;
@@ -1560,6 +1561,56 @@ pf_status ensure_device(pf_ctx *ctx) {
         if ((st = upload(ctx, &dn.yoff_br, ctx->yoff_br.data(), ctx->yoff_br.size()))) break;
         if ((st = upload(ctx, &dn.mis_ord, ctx->mis_ord.data(), ctx->mis_ord.size()))) break;
         if ((st = upload(ctx, &dn.mis_ord_cl, ctx->mis_ord_cl.data(), ctx->mis_ord_cl.size()))) break;
+        {
+            // fixed-point rows and branch terms (see DevNet); fma() as the
+            // device's own contraction, the same on every host
+            std::vector<double> bry(8 * size_t(std::max(1, nbranch)), 0.0), l1(nbus, 0.0);
+            std::vector<int> &ysc = ctx->ysc, yesc(dn.nnz);
+            ysc.assign(nbus, 0);
+            std::vector<int4> bryx(4 * size_t(std::max(1, nbranch)), int4{0, 0, 0, 0});
+            auto fx_scale = [](double sum) {  // units 2^-q that take `sum` to at most 2^58
+                int ex = 0;
+                if (!std::isfinite(sum)) return kFxNoScale;
+                std::frexp(sum, &ex);
+                return sum == 0.0 ? kFxRow : ex < -400 || ex > 400 ? kFxNoScale : kFxRow - ex;
+            };
+            for (int e = 0; e < nbranch; e++) {
+                const double den = std::fma(rr[e], rr[e], xx[e] * xx[e]);
+                const double g = rr[e] / den, b = -xx[e] / den, bc = std::fma(0.5, bb[e], b), t = tp[e];
+                double *o = &bry[8 * size_t(e)];
+                o[0] = g / (t * t);
+                o[1] = bc / (t * t);
+                o[2] = g;
+                o[3] = bc;
+                o[4] = -g / t;
+                o[5] = -b / t;
+                const int q = fx_scale(std::fabs(o[0]) + std::fabs(o[1]) + std::fabs(o[2]) + std::fabs(o[3]) +
+                                       std::fabs(o[4]) + std::fabs(o[5]));
+                for (int k = 0; k < 3 && q != kFxNoScale; k++) {
+                    const FxLimbs x = fx_split(fx_from_double(o[2 * k], q)), y = fx_split(fx_from_double(o[2 * k + 1], q));
+                    bryx[4 * size_t(e) + k] = int4{x.h, x.l, y.h, y.l};
+                }
+                bryx[4 * size_t(e) + 3] = int4{q, 0, 0, 0};
+                o[6] = 1.0 / xx[e];
+                if (!bst[e]) {
+                    std::fill(o, o + 8, 0.0);
+                    continue;
+                }
+                const double m = std::fabs(o[4]) + std::fabs(o[5]);
+                l1[bf[e]] += std::fabs(o[0]) + std::fabs(g / (t * t)) + std::fabs(b / (t * t)) +
+                             std::fabs(0.5 * bb[e] / (t * t)) + m;
+                l1[bt[e]] += std::fabs(o[2]) + std::fabs(g) + std::fabs(b) + std::fabs(0.5 * bb[e]) + m;
+            }
+            for (int i = 0; i < nbus; i++) {
+                ysc[i] = fx_scale(l1[i] + std::fabs(gs[i]) + std::fabs(bs[i]));
+                for (int p = ctx->rowptr[i]; p < ctx->rowptr[i + 1]; p++) yesc[p] = ysc[i];
+            }
+            if ((st = upload(ctx, &dn.bry, bry.data(), bry.size()))) break;
+            if ((st = upload(ctx, &dn.bryx, bryx.data(), bryx.size()))) break;
+            if ((st = upload(ctx, &dn.ysc, ysc.data(), ysc.size()))) break;
+            if ((st = upload(ctx, &dn.yesc, yesc.data(), yesc.size()))) break;
+            if ((st = dalloc(ctx, &dn.Yx, dn.nnz))) break;
+        }
         if ((st = dalloc(ctx, &dn.G, dn.nnz))) break;
         if ((st = dalloc(ctx, &dn.B, dn.nnz))) break;
         if ((st = dalloc(ctx, &dn.Bp, dn.nnz))) break;

@@ -320,6 +320,17 @@ struct DevNet {
     // number of its warp's lanes is active, so a warp's rows should be of
     // one length.
     int *mis_ord = nullptr, *mis_ord_cl = nullptr;
+    // Fixed-point form of the admittance rows (gbpf_fx.cuh): entry p in units
+    // 2^-ysc[i] of its row i (yesc[p] = ysc[i]) as limbs {G h, G l, B h, B l},
+    // written with G and B; the scale takes the sum of the magnitudes of every
+    // incident branch's terms and the shunt to at most 2^58 units, so any
+    // outage of the row's branches stays in range too.  bry[8 e ..]: branch
+    // e's terms G_ff, B_ff, G_tt, B_tt, G_ft, B_ft (pi model), 1/x, 0, all zero
+    // out of service; bryx[4 e
+    // ..]: the same three pairs as limbs in units 2^-q, then {q, 0, 0, 0}.
+    int *ysc = nullptr, *yesc = nullptr;
+    int4 *Yx = nullptr, *bryx = nullptr;
+    double *bry = nullptr;
 };
 
 struct DevCases {
@@ -432,7 +443,8 @@ struct pf_ctx {
     bool on_device = false;   // network and symbolic data uploaded
     std::vector<int> ydiag, inc_ptr, inc_br, inc_side, inc_pos, br_pos, yoff_br;
     std::vector<int4> yoff;
-    std::vector<int> mis_ord, mis_ord_cl;
+    std::vector<int> mis_ord, mis_ord_cl, ysc;
+    std::vector<char> bridge;  // per branch: its outage splits the grid (on first use)
     int device = 0;
     int num_sms = 0;
     size_t smem_optin = 0;
@@ -473,6 +485,9 @@ cudaError_t launch_assemble_slots(const DevNet &dn, const DevCases &dc, const De
                                   double *A, cudaStream_t s, int ninst = -1);
 cudaError_t launch_branch_flows(const DevNet &dn, const DevCases &dc, const double *vm, const double *va,
                                 int ncase, double *flows, double *loss, cudaStream_t s);
+// e + jf of every case's state in fixed point (gbpf_fx.cuh) into the first
+// half of its ef region [4 nbus]; kFxNone where a voltage is out of range.
+cudaError_t launch_polar(const DevNet &dn, int ncase, const double *vm, const double *va, double *ef, cudaStream_t s);
 struct FactorSync {
     unsigned *done = nullptr;  // [ninst][n]
     unsigned *sync = nullptr;  // [0] column counter, [1] abort flag

@@ -28,58 +28,57 @@ namespace {
 
 // ------------------------------------------------------------ Section III.A
 
+__device__ __forceinline__ int4 fx_entry(double g, double b, int q) {
+    if (q == kFxNoScale) return make_int4(0, 0, 0, 0);
+    const FxLimbs x = fx_split(fx_from_double(g, q)), y = fx_split(fx_from_double(b, q));
+    return make_int4(x.h, x.l, y.h, y.l);
+}
+
 // FormMatrixA (Section III.A), one thread per entry of Y = G + jB: threads
 // [0, nbus) the diagonal of bus i -- the pi-model self terms of its
 // in-service incident branches (incidence order: ascending branch index)
 // plus the bus shunt -- and threads [nbus, nbus + noff) one off-diagonal
 // entry each, the negated series admittances of the in-service branches
-// between its two buses (ascending branch index).  Every entry is formed in
-// registers and written once; a diagonal thread reads the indices of four
-// incident branches at a time before their parameters, so a bus of degree
-// up to four costs three dependent round trips to memory.  Also writes the
-// XB B' (1/x weights) on the same pattern.
+// between its two buses (ascending branch index).  The branches' terms come
+// from the table bry (zero rows out of service).  Every entry is formed in
+// registers and written once, with the XB B' (1/x weights) on the same pattern
+// and the entry's fixed-point form.  Bound by latency: the indices of four
+// incident branches are read before their terms, three round trips to memory
+// (with the terms formed here, four FP64 divisions a branch in a row, a launch
+// took 18 to 22 us at any size up to 10,000 buses).
 __device__ __forceinline__ void ybus_entry(const DevNet &dn, int t) {
     if (t < dn.nbus) {
         const int i = t, q1 = dn.inc_ptr[i + 1];
+        const double gs = dn.gs[i], bs = dn.bs[i];
+        const int d = dn.ydiag[i];
         double gd = 0.0, bd = 0.0, bpd = 0.0;
         for (int q = dn.inc_ptr[i]; q < q1; q += 4) {
-            int e[4], sd[4], on[4];
-            double r[4], x[4], b[4], tp[4];
+            const double2 *y[4];
+            double2 self[4], x[4];
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                e[u] = q + u < q1 ? dn.inc_br[q + u] : -1;
-                sd[u] = q + u < q1 ? dn.inc_side[q + u] : 0;
-            }
+            for (int u = 0; u < 4; u++)
+                y[u] = reinterpret_cast<const double2 *>(dn.bry + 8LL * (q + u < q1 ? dn.inc_br[q + u] : 0)) +
+                       (q + u < q1 ? dn.inc_side[q + u] : 0);
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                on[u] = 0;
-                if (e[u] >= 0) {
-                    on[u] = dn.bstatus[e[u]];
-                    r[u] = dn.br[e[u]];
-                    x[u] = dn.bx[e[u]];
-                    b[u] = dn.bb[e[u]];
-                    tp[u] = dn.btap[e[u]];
+            for (int u = 0; u < 4; u++)
+                if (q + u < q1) {
+                    self[u] = y[u][0];
+                    x[u] = y[u][3 - (q + u < q1 ? dn.inc_side[q + u] : 0)];
                 }
-            }
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                if (!on[u]) continue;
-                const double den = r[u] * r[u] + x[u] * x[u];
-                const double ys_re = r[u] / den, ys_im = -x[u] / den;
-                if (sd[u] == 0) {
-                    gd += ys_re / (tp[u] * tp[u]);
-                    bd += (ys_im + 0.5 * b[u]) / (tp[u] * tp[u]);
-                } else {
-                    gd += ys_re;
-                    bd += ys_im + 0.5 * b[u];
+            for (int u = 0; u < 4; u++)
+                if (q + u < q1) {
+                    gd += self[u].x;
+                    bd += self[u].y;
+                    bpd += x[u].x;
                 }
-                bpd += 1.0 / x[u];
-            }
         }
-        const int d = dn.ydiag[i];
-        dn.G[d] = gd + dn.gs[i];
-        dn.B[d] = bd + dn.bs[i];
+        gd += gs;
+        bd += bs;
+        dn.G[d] = gd;
+        dn.B[d] = bd;
         dn.Bp[d] = bpd;
+        dn.Yx[d] = fx_entry(gd, bd, dn.yesc[d]);
         return;
     }
     const int k = t - dn.nbus;
@@ -87,18 +86,16 @@ __device__ __forceinline__ void ybus_entry(const DevNet &dn, int t) {
     const int4 o = dn.yoff[k];
     double g = 0.0, bo = 0.0, bp = 0.0;
     for (int q = o.y; q < o.z; q++) {
-        const int e = dn.yoff_br[q];
-        if (!dn.bstatus[e]) continue;
-        const double r = dn.br[e], x = dn.bx[e], tp = dn.btap[e];
-        const double den = r * r + x * x;
-        const double ys_re = r / den, ys_im = -x / den;
-        g -= ys_re / tp;
-        bo -= ys_im / tp;
-        bp -= 1.0 / x;
+        const double2 *y = reinterpret_cast<const double2 *>(dn.bry + 8LL * dn.yoff_br[q]);
+        const double2 m = y[2];
+        g += m.x;
+        bo += m.y;
+        bp -= y[3].x;
     }
     dn.G[o.x] = g;
     dn.B[o.x] = bo;
     dn.Bp[o.x] = bp;
+    dn.Yx[o.x] = fx_entry(g, bo, dn.yesc[o.x]);
 }
 
 __global__ void k_ybus(DevNet dn) {
@@ -754,6 +751,11 @@ __global__ void __launch_bounds__(kFactorThreads)
 // Flows of branch k in case c: S_f = V_f conj(I_f), S_t = V_t conj(I_t) with
 // the pi model (series y = 1/(r + jx), charging jb/2 at each end, tap t on
 // the from side); zero for the case's outage and out-of-service branches.
+// From the end voltages in fixed point and the branch's terms (units 2^-q,
+// their sum at most 2^58): I_f and I_t in units 2^-(q + 1), the powers in
+// units 2^-(q + 2).  A branch with an end outside the fixed-point range takes
+// the FP64 form.  Both ends' voltages are formed per branch rather than once
+// per bus: the call needs no scratch that calls on other streams share.
 __global__ void k_branch_flows(DevNet dn, DevCases dc, const double *vm, const double *va, int ncase,
                                double *flows) {
     const long long total = (long long)ncase * dn.nbr;
@@ -767,22 +769,52 @@ __global__ void k_branch_flows(DevNet dn, DevCases dc, const double *vm, const d
         }
         const int f = dn.bf[k], t = dn.bt[k];
         const double *vmc = vm + (long long)c * dn.nbus, *vac = va + (long long)c * dn.nbus;
+        const int4 vf = fx_polar_any(vmc[f], vac[f]), vt = fx_polar_any(vmc[t], vac[t]);
+        if (vf.x != kFxNone && vt.x != kFxNone && dn.bryx[4 * k + 3].x != kFxNoScale) {
+            const int4 yf = dn.bryx[4 * k], yt = dn.bryx[4 * k + 1], ym = dn.bryx[4 * k + 2];
+            const int q = dn.bryx[4 * k + 3].x + 2;
+            auto current = [](const int4 &y, const int4 &v, const int4 &z, const int4 &w, long long &re, long long &im) {
+                FxAcc a{0, 0}, b{0, 0};
+                fx_mac(a, y.x, y.y, v.x, v.y);
+                fx_mac(a, -y.z, -y.w, v.z, v.w);
+                fx_mac(a, z.x, z.y, w.x, w.y);
+                fx_mac(a, -z.z, -z.w, w.z, w.w);
+                fx_mac(b, y.x, y.y, v.z, v.w);
+                fx_mac(b, y.z, y.w, v.x, v.y);
+                fx_mac(b, z.x, z.y, w.z, w.w);
+                fx_mac(b, z.z, z.w, w.x, w.y);
+                re = fx_sum<3>(a);
+                im = fx_sum<3>(b);
+            };
+            long long fr, fi, tr, ti;
+            current(yf, vf, ym, vt, fr, fi);
+            current(yt, vt, ym, vf, tr, ti);
+            const double pf = fx_to_double(fx_power(false, vf, fr, fi), q), qf = fx_to_double(fx_power(true, vf, fr, fi), q);
+            const double pt = fx_to_double(fx_power(false, vt, tr, ti), q), qt = fx_to_double(fx_power(true, vt, tr, ti), q);
+            if (reinterpret_cast<uintptr_t>(flows) & 15) {  // the caller's array may be 8-byte aligned only
+                o[0] = pf; o[1] = qf; o[2] = pt; o[3] = qt;
+            } else {
+                reinterpret_cast<double2 *>(o)[0] = make_double2(pf, qf);
+                reinterpret_cast<double2 *>(o)[1] = make_double2(pt, qt);
+            }
+            continue;
+        }
         double sf, cf, st, ct;
         sincos(vac[f], &sf, &cf);
         sincos(vac[t], &st, &ct);
-        const double ef = vmc[f] * cf, ff = vmc[f] * sf, et = vmc[t] * ct, ft = vmc[t] * st;
+        const double fe = vmc[f] * cf, ff = vmc[f] * sf, et = vmc[t] * ct, ft = vmc[t] * st;
         const double r = dn.br[k], x = dn.bx[k], den = r * r + x * x;
         const double g = r / den, b = -x / den, bc = 0.5 * dn.bb[k];
         const double tap = dn.btap[k] != 0.0 ? dn.btap[k] : 1.0;
         // I_f = ((g + j(b + bc)) / t^2) V_f - ((g + jb) / t) V_t
         const double gff = g / (tap * tap), bff = (b + bc) / (tap * tap), gft = -g / tap, bft = -b / tap;
-        const double ifr = gff * ef - bff * ff + gft * et - bft * ft;
-        const double ifi = gff * ff + bff * ef + gft * ft + bft * et;
+        const double ifr = gff * fe - bff * ff + gft * et - bft * ft;
+        const double ifi = gff * ff + bff * fe + gft * ft + bft * et;
         // I_t = -((g + jb) / t) V_f + (g + j(b + bc)) V_t
-        const double itr = gft * ef - bft * ff + g * et - (b + bc) * ft;
-        const double iti = gft * ff + bft * ef + g * ft + (b + bc) * et;
-        o[0] = ef * ifr + ff * ifi;
-        o[1] = ff * ifr - ef * ifi;
+        const double itr = gft * fe - bft * ff + g * et - (b + bc) * ft;
+        const double iti = gft * ff + bft * fe + g * ft + (b + bc) * et;
+        o[0] = fe * ifr + ff * ifi;
+        o[1] = ff * ifr - fe * ifi;
         o[2] = et * itr + ft * iti;
         o[3] = ft * itr - et * iti;
     }
@@ -925,43 +957,81 @@ __global__ void k_lowrank_k(DevMat m, DevNet dn, DevCases dc, int which, const T
 
 // ------------------------------------------------------------ Section II.A
 
-__global__ void k_polar_to_rect(int nbus, int ncase, const double *vm, const double *va,
-                                double *ef) {
+// e + jf of every bus of every case in fixed point, ef[c * st + i].
+__global__ void k_polar_to_rect(int nbus, int ncase, const double *vm, const double *va, int4 *ef, long long st) {
     const long long total = (long long)ncase * nbus;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         const long long c = idx / nbus;
-        const int i = int(idx % nbus);
-        double s, co;
-        sincos(va[idx], &s, &co);
-        ef[c * 4 * nbus + i] = vm[idx] * co;
-        ef[c * 4 * nbus + nbus + i] = vm[idx] * s;
+        ef[c * st + (idx - c * nbus)] = fx_polar_any(vm[idx], va[idx]);
     }
 }
 
-__global__ void k_mismatch_rows(DevNet dn, DevCases dc, const double *ef, double *dp, double *dq,
-                                double *maxmis) {
+// The FP64 form of (P, Q) at bus i of one case from its polar state, for rows
+// with a voltage outside the fixed-point range.
+__device__ __noinline__ void polar_injection(const DevNet &dn, int i, int outage, const double *vm, const double *va,
+                                             double &P, double &Q) {
+    double s, c, ir = 0.0, ii = 0.0;
+    for (int p = dn.rowptr[i]; p < dn.rowptr[i + 1]; p++) {
+        const int k = dn.col[p];
+        double g = dn.G[p], b = dn.B[p];
+        if (outage >= 0 && dn.bstatus[outage]) {
+            const int f = dn.bf[outage], t = dn.bt[outage];
+            const double *y = dn.bry + 8LL * outage;
+            if ((i == f || i == t) && (k == f || k == t)) {
+                const int o = i != k ? 4 : (i == f ? 0 : 2);
+                g -= y[o];
+                b -= y[o + 1];
+            }
+        }
+        sincos(va[k], &s, &c);
+        const double e = vm[k] * c, f = vm[k] * s;
+        ir += g * e - b * f;
+        ii += g * f + b * e;
+    }
+    sincos(va[i], &s, &c);
+    P = vm[i] * c * ir + vm[i] * s * ii;
+    Q = vm[i] * s * ir - vm[i] * c * ii;
+}
+
+// spec - value of a fixed-point power in units 2^-q.
+__device__ __forceinline__ double fx_mismatch(double spec, long long value, int q) {
+    return fx_fits(spec, q) ? fx_to_double(fx_from_double(spec, q) - value, q) : spec - fx_to_double(value, q);
+}
+
+// 10,000 buses x 256 cases: 228 us in FP64.
+__global__ void k_mismatch_rows(DevNet dn, DevCases dc, const double *vm, const double *va, const int4 *ef,
+                                long long st, double *dp, double *dq, double *maxmis) {
     const int c = blockIdx.y;
     const int nbus = dn.nbus;
-    const double *e = ef + (long long)c * 4 * nbus;
-    const double *f = e + nbus;
+    const int4 *v = ef + c * st;
     const int outage = dc.outage[c];
-    double mx = 0.0;
+    unsigned long long mx = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nbus; i += gridDim.x * blockDim.x) {
-        double P, Q;
-        bus_injection(dn, i, outage, e, f, P, Q);
-        const int t = dn.btype[i];
+        const int t = dn.btype[i], q = dn.ysc[i] + 2;
         const long long idx = (long long)c * nbus + i;
-        const double a = (t != PF_BUS_SLACK) ? dc.Psp[idx] - P : 0.0;
-        const double b = (t == PF_BUS_PQ) ? dc.Qsp[idx] - Q : 0.0;
+        long long ir, ii;
+        double a = 0.0, b = 0.0;
+        if (fx_bus_current<true>(dn, i, outage, v, 1, ir, ii)) {
+            if (t != PF_BUS_SLACK) a = fx_mismatch(dc.Psp[idx], fx_power(false, v[i], ir, ii), q);
+            if (t == PF_BUS_PQ) b = fx_mismatch(dc.Qsp[idx], fx_power(true, v[i], ir, ii), q);
+        } else {
+            double P, Q;
+            polar_injection(dn, i, outage, vm + (long long)c * nbus, va + (long long)c * nbus, P, Q);
+            if (t != PF_BUS_SLACK) a = dc.Psp[idx] - P;
+            if (t == PF_BUS_PQ) b = dc.Qsp[idx] - Q;
+        }
         dp[idx] = a;
         dq[idx] = b;
-        double l = fmax(fabs(a), fabs(b));
-        if (a != a || b != b) l = __longlong_as_double(0x7ff8000000000000ll);
-        mx = nan_max(mx, l);
+        const unsigned long long ka = abs_key(a), kb = abs_key(b), k = ka > kb ? ka : kb;
+        mx = k > mx ? k : mx;
     }
-    mx = warp_max(mx);
-    if ((threadIdx.x & 31) == 0) atomic_max_nonneg(maxmis + c, mx);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_xor_sync(0xffffffffu, mx, o);
+        mx = w > mx ? w : mx;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned long long *>(maxmis + c), mx);
 }
 
 int grid_for(long long total, int threads) {
@@ -1270,15 +1340,23 @@ cudaError_t launch_selftest_sweep(const DevMat &m, int prec, const void *F, cons
     return cudaGetLastError();
 }
 
+// e + jf of every case's state into the first half of its ef region.
+cudaError_t launch_polar(const DevNet &dn, int ncase, const double *vm, const double *va, double *ef, cudaStream_t s) {
+    k_polar_to_rect<<<grid_for((long long)ncase * dn.nbus, 256), 256, 0, s>>>(
+        dn.nbus, ncase, vm, va, reinterpret_cast<int4 *>(ef), 2LL * dn.nbus);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_mismatch(const DevNet &dn, const DevCases &dc, const double *vm, const double *va,
                             double *dp, double *dq, double *maxmis, double *ef, int ncase,
                             cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(maxmis, 0, sizeof(double) * ncase, s);
     if (e != cudaSuccess) return e;
-    k_polar_to_rect<<<grid_for((long long)ncase * dn.nbus, 256), 256, 0, s>>>(dn.nbus, ncase, vm,
-                                                                              va, ef);
+    e = launch_polar(dn, ncase, vm, va, ef, s);
+    if (e != cudaSuccess) return e;
     dim3 grid((dn.nbus + 255) / 256, ncase);
-    k_mismatch_rows<<<grid, 256, 0, s>>>(dn, dc, ef, dp, dq, maxmis);
+    k_mismatch_rows<<<grid, 256, 0, s>>>(dn, dc, vm, va, reinterpret_cast<const int4 *>(ef), 2LL * dn.nbus, dp, dq,
+                                         maxmis);
     return cudaGetLastError();
 }
 

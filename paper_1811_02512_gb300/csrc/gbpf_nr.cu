@@ -86,66 +86,109 @@ __global__ void __launch_bounds__(512, C == 1 ? 2 : 1) k_adjoint(NrArgs a, int f
 }
 
 // Objective J = sum_i (V_i - 1)^2 + sum_i P_i (total active losses) of case c
-// (one block per case) and its gradient with respect to every bus angle and
-// magnitude: dJ/dtheta_k = sum_l dP_l/dtheta_k, dJ/dV_k = 2 (V_k - 1) +
-// sum_l dP_l/dV_k, summed over every row l including the slack.
-__global__ void __launch_bounds__(512) k_objective(DevNet dn, DevCases dc, const double *vm,
-                                                   const double *va, double *ef, double *Jv,
-                                                   double *gva, double *gvm) {
-    __shared__ double red[33];
-    const int c = blockIdx.x;
-    const int nbus = dn.nbus;
-    const double *v = vm + (long long)c * nbus;
-    const double *th = va + (long long)c * nbus;
-    double *e = ef + (long long)c * 4 * nbus;
-    double *f = e + nbus;
-    double *P = e + 2 * nbus;
-    double *Q = e + 3 * nbus;
+// and its gradient with respect to every bus angle and magnitude.  The
+// admittance matrix is symmetric (no phase shift), so with V = e + jf the sum
+// of the injections is e'Ge + f'Gf -- the susceptances cancel -- and
+//   dJ/dtheta_k = 2 (e_k (Gf)_k - f_k (Ge)_k),
+//   dJ/dV_k = 2 (V_k - 1) + 2 (e_k (Ge)_k + f_k (Gf)_k) / V_k:
+// six integer multiply-adds an entry in fixed point (gbpf_fx.cuh) where the
+// sums of dP_l/dtheta_k and dP_l/dV_k over the rows l took a dozen FP64
+// operations and two divisions, and no cancelling terms.  A row with a
+// voltage outside the fixed-point range takes the FP64 form.  Block b of a
+// case writes its part of J to part[b]; blocks of 256 buses, so a single
+// case spreads over the GPU.
+__global__ void __launch_bounds__(256) k_objective(DevNet dn, DevCases dc, const double *vm, const double *va,
+                                                   double *ef, double *gva, double *gvm) {
+    __shared__ double red[8];
+    const int nbus = dn.nbus, nblk = (nbus + 255) / 256;
+    const int c = int(blockIdx.x / nblk), i = int(blockIdx.x % nblk) * 256 + int(threadIdx.x);
+    const int4 *u = reinterpret_cast<const int4 *>(ef + (long long)c * 4 * nbus);
     const int outage = dc.outage[c];
-    for (int i = threadIdx.x; i < nbus; i += blockDim.x) {
-        double s, co;
-        sincos(th[i], &s, &co);
-        e[i] = v[i] * co;
-        f[i] = v[i] * s;
-    }
-    __syncthreads();
     double part = 0.0;
-    for (int i = threadIdx.x; i < nbus; i += blockDim.x) {
-        double p, q;
-        bus_injection(dn, i, outage, e, f, p, q);
-        P[i] = p;
-        Q[i] = q;
-        part += (v[i] - 1.0) * (v[i] - 1.0) + p;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < nbus; k += blockDim.x) {
-        double gt = 0.0, gv = 2.0 * (v[k] - 1.0);
-        for (int p = dn.rowptr[k]; p < dn.rowptr[k + 1]; p++) {
-            const int l = dn.col[p];
-            double G, B;
-            y_entry(dn, outage, l, k, p, G, B);  // Y is symmetric: Y_lk at row k's slot
-            if (l != k) {
-                const B2<double> J = jac_off(G, B, e[l], f[l], e[k], f[k], v[k], false, false);
-                gt += J.a;
-                gv += J.b;
-            } else {
-                const B2<double> J = jac_diag(G, B, P[k], Q[k], v[k], false);
-                gt += J.a;
-                gv += J.b;
+    if (i < nbus) {
+        const long long idx = (long long)c * nbus + i;
+        const double v = vm[idx];
+        const int4 w = u[i];
+        bool ok = w.x != kFxNone && fx_vm_ok(v) && dn.ysc[i] != kFxNoScale;
+        FxAcc a{0, 0}, b{0, 0};  // (Ge)_i, (Gf)_i
+        const int pe = dn.rowptr[i + 1];
+        for (int p = dn.rowptr[i]; p < pe; p += 4) {
+            int4 x[4];
+            int2 g[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                x[q] = u[p + q < pe ? dn.col[p + q] : i];
+                g[q] = p + q < pe ? *reinterpret_cast<const int2 *>(dn.Yx + p + q) : make_int2(0, 0);
             }
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                ok &= x[q].x != kFxNone;
+                fx_mac(a, g[q].x, g[q].y, x[q].x, x[q].y);
+                fx_mac(b, g[q].x, g[q].y, x[q].z, x[q].w);
+            }
+            fx_carry(a);
+            fx_carry(b);
         }
-        gva[(long long)c * nbus + k] = gt;
-        gvm[(long long)c * nbus + k] = gv;
+        const bool at_outage = outage >= 0 && dn.bstatus[outage] && (i == dn.bf[outage] || i == dn.bt[outage]);
+        double gt, gv, pw;
+        if (ok) {
+            if (at_outage) {
+                const int o = i == dn.bf[outage] ? dn.bt[outage] : dn.bf[outage];
+                const double *y = dn.bry + 8LL * outage;
+                const FxLimbs gs = fx_split(-fx_from_double(y[i == dn.bf[outage] ? 0 : 2], dn.ysc[i]));
+                const FxLimbs gm = fx_split(-fx_from_double(y[4], dn.ysc[i]));
+                const int4 x = u[o];
+                fx_mac(a, gs.h, gs.l, w.x, w.y);
+                fx_mac(a, gm.h, gm.l, x.x, x.y);
+                fx_mac(b, gs.h, gs.l, w.z, w.w);
+                fx_mac(b, gm.h, gm.l, x.z, x.w);
+            }
+            const long long ge = fx_sum<3>(a), gf = fx_sum<3>(b);
+            const int q = dn.ysc[i] + 2;
+            const long long s = fx_power(false, w, ge, gf);  // e Ge + f Gf
+            const long long t = -fx_power(true, w, ge, gf);  // e Gf - f Ge
+            gt = fx_to_double(t, q - 1);
+            pw = fx_to_double(s, q);
+            gv = 2.0 * (v - 1.0) + fx_over_v(s, q - 1, fx_recip(fx_from_double(v, kFxV)));
+        } else {
+            double ge = 0.0, gf = 0.0, sn, cs;
+            for (int p = dn.rowptr[i]; p < pe; p++) {
+                const int k = dn.col[p];
+                double g, bb;
+                y_entry(dn, outage, i, k, p, g, bb);
+                sincos(va[(long long)c * nbus + k], &sn, &cs);
+                ge += g * (vm[(long long)c * nbus + k] * cs);
+                gf += g * (vm[(long long)c * nbus + k] * sn);
+            }
+            sincos(va[idx], &sn, &cs);
+            gt = 2.0 * v * (cs * gf - sn * ge);
+            pw = v * (cs * ge + sn * gf);
+            gv = 2.0 * (v - 1.0) + 2.0 * (cs * ge + sn * gf);
+        }
+        gva[idx] = gt;
+        gvm[idx] = gv;
+        part = (v - 1.0) * (v - 1.0) + pw;
     }
-    // block sum of the objective (fixed order: warp shuffles then warps)
+    // block sum (fixed order: warp shuffles, then warps)
     for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = part;
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0.0;
-        for (int w = 0; w < int(blockDim.x >> 5); w++) s += red[w];
-        Jv[c] = s;
+        for (int w = 0; w < 8; w++) s += red[w];
+        ef[(long long)c * 4 * nbus + 2 * nbus + blockIdx.x % nblk] = s;
     }
+}
+
+// J of case c from its blocks' parts, in block order.
+__global__ void k_objective_sum(int nbus, int nblk, int ncase, const double *ef, double *Jv) {
+    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (c >= ncase) return;
+    const double *p = ef + (long long)c * 4 * nbus + 2 * nbus;
+    double s = 0.0;
+    for (int b = lane; b < nblk; b += 32) s += p[b];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) Jv[c] = s;
 }
 
 template <int C, class... Args>
@@ -316,7 +359,11 @@ cudaError_t launch_nr(const NrLaunch &L, cudaStream_t s) {
 
 cudaError_t launch_objective(const DevNet &dn, const DevCases &dc, const double *vm, const double *va,
                              double *ef, double *J, double *gva, double *gvm, cudaStream_t s) {
-    k_objective<<<dc.ncase, 512, 0, s>>>(dn, dc, vm, va, ef, J, gva, gvm);
+    cudaError_t e = launch_polar(dn, dc.ncase, vm, va, ef, s);
+    if (e != cudaSuccess) return e;
+    const int nblk = (dn.nbus + 255) / 256;  // parts of J per case, after the case's e + jf
+    k_objective<<<unsigned(nblk) * unsigned(dc.ncase), 256, 0, s>>>(dn, dc, vm, va, ef, gva, gvm);
+    k_objective_sum<<<(dc.ncase + 3) / 4, 128, 0, s>>>(dn.nbus, nblk, dc.ncase, ef, J);
     return cudaGetLastError();
 }
 
