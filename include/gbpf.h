@@ -132,8 +132,9 @@ typedef struct {
  * step of all blocks followed by a cluster barrier, and the narrow top of
  * the tree is solved with the explicit inverse of its block of L (three
  * steps in all); it needs the factors' programs to fit in shared memory.
- * AUTO picks BLOCK; LANES and CLUSTER fall back to BLOCK where they do not
- * apply. */
+ * AUTO takes the context's tuning; where that names no engine, cluster size,
+ * tail form or block size, CLUSTER where it applies and else BLOCK.  LANES
+ * and CLUSTER fall back to BLOCK where they do not apply. */
 enum { PF_ENGINE_AUTO = 0, PF_ENGINE_BLOCK = 1, PF_ENGINE_LANES = 2, PF_ENGINE_CLUSTER = 3 };
 
 /* Kernel mappings of a context, chosen by pf_autotune (or set directly with

@@ -296,29 +296,42 @@ __device__ __forceinline__ void cl_step(const ClSmem &S, int4 si) {
     }
 }
 
-// Mismatch of one half-iteration (as k_fdpf's cluster_mismatch): the CTA's
-// bus slice forms e + jf, then (after a cluster barrier) the currents of its
-// rows; dP/V (which = 0) or dQ/V (which = 1) goes straight into the owner's
+// The cluster maximum of the CTAs' keys mx (slot `which` of each CTA's mkey).
+template <int C>
+__device__ __forceinline__ double cl_exchange_max(unsigned long long mx, int which, double *red,
+                                                  unsigned long long *mkey, const uint32_t *kbase) {
+    mx = block_max_key(mx, red);
+    // the CTAs' maxima are exchanged as integer keys through distributed
+    // shared memory: slot `which` of each CTA's mkey
+    if (threadIdx.x == 0) mkey[which] = mx;
+    cl_barrier();
+    unsigned long long k = 0;
+    if (threadIdx.x < C) k = ld_cl_u64(kbase[threadIdx.x] + 8u * unsigned(which));
+    for (int o = C / 2; o > 0; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, k, o);
+        k = u > k ? u : k;
+    }
+    k = __shfl_sync(0xffffffffu, k, 0);
+    if ((threadIdx.x >> 5) == 0 && (threadIdx.x & 31) == 0) red[32] = __longlong_as_double(static_cast<long long>(k));
+    __syncthreads();
+    return red[32];
+}
+
+// Mismatch of one half-iteration (as k_fdpf's cluster_mismatch) from the
+// e + jf written with the state: after a cluster barrier the currents of the
+// CTA's rows; dP/V (which = 0) or dQ/V (which = 1) goes straight into the owner's
 // vector slot of the matrix (rhsref: owner << 16 | word, -1 for a bus
 // outside the matrix).  Returns the cluster maximum of the half-iteration's
-// part (full: of both parts).  ef_ready: the slice's e + jf were already
-// written with the state (by the update that produced it).
+// part (full: of both parts).
 template <int C>
 __device__ double cl_mismatch(const ClRun &a, int rank, int which, const uint32_t *xbase, double *red,
-                              unsigned long long *mkey, const uint32_t *kbase, bool full, bool ef_ready) {
+                              unsigned long long *mkey, const uint32_t *kbase, bool full) {
     const DevNet &dn = a.dn;
     const int nbus = dn.nbus;
     const int slice = (nbus + C - 1) / C;
     const int i0 = rank * slice, i1 = min(nbus, i0 + slice);
     double *e = a.ef;
     double *f = e + nbus;
-    const double *cs = e + 2 * nbus;
-    const double *sn = e + 3 * nbus;
-    if (!ef_ready)
-        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-            e[i] = a.vm[i] * cs[i];
-            f[i] = a.vm[i] * sn[i];
-        }
     cl_barrier_global();
     const int *rhsref = a.m[which].rhsref;
     const bool wantP = full || which == 0, wantQ = full || which == 1;
@@ -337,21 +350,42 @@ __device__ double cl_mismatch(const ClRun &a, int rank, int which, const uint32_
         const int r = rhsref[i];
         if (r >= 0) st_cl(xbase[which * C + (r >> 16)] + 8u * unsigned(r & 0xffff), (which == 0 ? dP : dQ) * a.iv[i]);
     }
-    mx = block_max_key(mx, red);
-    // the CTAs' maxima are exchanged as integer keys through distributed
-    // shared memory: slot `which` of each CTA's mkey
-    if (threadIdx.x == 0) mkey[which] = mx;
-    cl_barrier();
-    unsigned long long k = 0;
-    if (threadIdx.x < C) k = ld_cl_u64(kbase[threadIdx.x] + 8u * unsigned(which));
-    for (int o = C / 2; o > 0; o >>= 1) {
-        const unsigned long long u = __shfl_xor_sync(0xffffffffu, k, o);
-        k = u > k ? u : k;
+    return cl_exchange_max<C>(mx, which, red, mkey, kbase);
+}
+
+// The fixed-point form (as k_fdpf's cluster_mismatch_fx): left = this thread
+// saw a bus leave the fixed-point range; the maximum is then the all-ones key.
+template <int C>
+__device__ double cl_mismatch_fx(const ClRun &a, int rank, int which, const uint32_t *xbase, double *red,
+                                 unsigned long long *mkey, const uint32_t *kbase, bool full, bool left) {
+    const DevNet &dn = a.dn;
+    const int nbus = dn.nbus;
+    const int slice = (nbus + C - 1) / C;
+    const int i0 = rank * slice, i1 = min(nbus, i0 + slice);
+    const int4 *ef = reinterpret_cast<const int4 *>(a.ef);
+    const long long *iv = reinterpret_cast<const long long *>(a.iv);
+    cl_barrier_global();
+    const int *rhsref = a.m[which].rhsref;
+    const bool wantP = full || which == 0, wantQ = full || which == 1;
+    unsigned long long mx = left ? ~0ull : 0ull;
+    for (int q = i0 + threadIdx.x; q < i1; q += blockDim.x) {
+        const int i = C == kClCtas ? dn.mis_ord_cl[q] : q;  // a warp's rows of one length
+        const int t = dn.btype[i], sc = dn.ysc[i] + 2, r = rhsref[i];
+        const double psp = wantP ? a.dc.Psp[i] : 0.0, qsp = wantQ ? a.dc.Qsp[i] : 0.0;
+        const int4 v = ef[i];
+        const long long ivi = iv[i];
+        long long ir, ii;
+        fx_bus_current<false>(dn, i, -1, ef, 1, ir, ii);
+        long long dP = 0, dQ = 0;
+        if (wantP && t != PF_BUS_SLACK) dP = fx_from_double(psp, sc) - fx_power(false, v, ir, ii);
+        if (wantQ && t == PF_BUS_PQ) dQ = fx_from_double(qsp, sc) - fx_power(true, v, ir, ii);
+        const long long ap = dP < 0 ? -dP : dP, aq = dQ < 0 ? -dQ : dQ;
+        const unsigned long long key = abs_key(fx_to_double(ap > aq ? ap : aq, sc));
+        mx = key > mx ? key : mx;
+        if (r >= 0)
+            st_cl(xbase[which * C + (r >> 16)] + 8u * unsigned(r & 0xffff), fx_over_v(which == 0 ? dP : dQ, sc, ivi));
     }
-    k = __shfl_sync(0xffffffffu, k, 0);
-    if ((threadIdx.x >> 5) == 0 && (threadIdx.x & 31) == 0) red[32] = __longlong_as_double(static_cast<long long>(k));
-    __syncthreads();
-    return red[32];
+    return cl_exchange_max<C>(mx, which, red, mkey, kbase);
 }
 
 template <int C>
@@ -382,8 +416,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
     {  // the admittance matrix is read every half-iteration: start it towards the L2
         const int part = rank * kClThreads + int(threadIdx.x), parts = C * kClThreads;
         l2_prefetch(dn.col, sizeof(int) * size_t(dn.nnz), part, parts);
-        l2_prefetch(dn.G, sizeof(double) * size_t(dn.nnz), part, parts);
-        l2_prefetch(dn.B, sizeof(double) * size_t(dn.nnz), part, parts);
+        l2_prefetch(dn.Yx, sizeof(int4) * size_t(dn.nnz), part, parts);
     }
     __syncthreads();
     for (int w = 0; w < 2; w++) {
@@ -410,6 +443,9 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
     double *vm = a.vm, *va = a.va, *iv = a.iv;
     double *ef = a.ef;  // e, f, then cos and sin of the angles
     double *cs = a.ef + 2 * nbus, *sn = cs + nbus;
+    int4 *efx = reinterpret_cast<int4 *>(a.ef);  // e + jf and 1/V in fixed point
+    long long *ivx = reinterpret_cast<long long *>(a.iv);
+    bool left = false;  // a bus of this thread is out of the fixed-point range
     int status = PF_ERR_NOT_CONVERGED;
     if (a.fs0[0] != PF_OK) status = a.fs0[0];
     else if (a.fs1[0] != PF_OK) status = a.fs1[0];
@@ -421,15 +457,36 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
             vm[i] = (t == PF_BUS_PQ) ? 1.0 : dn.vset[i];
             va[i] = (t == PF_BUS_SLACK) ? dn.va0[i] : 0.0;
         }
-        sincos(va[i], &sn[i], &cs[i]);
-        iv[i] = 1.0 / vm[i];
-        ef[i] = vm[i] * cs[i];
-        ef[nbus + i] = vm[i] * sn[i];
+        if (fx_state_ok(dn, i, vm[i], va[i], a.dc.Psp[i], a.dc.Qsp[i])) {
+            efx[i] = fx_polar(vm[i], va[i]);
+            ivx[i] = fx_recip(fx_from_double(vm[i], kFxV));
+        } else {
+            left = true;
+        }
     }
     // e + jf of every bus is written where the state changes (here, and in
-    // the updates below), so the mismatch needs no pass of its own
-    bool rotated = false;
+    // the updates below), so the mismatch needs no pass of its own; in fixed
+    // point while every bus is in its range, else in FP64 with cached cos and
+    // sin of the angles (as k_fdpf)
+    bool rotated = false, fx = true;
+    auto enter_fp64 = [&]() {
+        fx = false;
+        rotated = false;
+        cl_barrier_global();  // e + jf and 1/V change their form
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+            sincos(va[i], &sn[i], &cs[i]);
+            iv[i] = 1.0 / vm[i];
+            ef[i] = vm[i] * cs[i];
+            ef[nbus + i] = vm[i] * sn[i];
+        }
+    };
     auto exact_check = [&](int which) {
+        if (fx) {
+            if (rotated)
+                for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) efx[i] = fx_polar(vm[i], va[i]);
+            rotated = false;
+            return cl_mismatch_fx<C>(a, rank, which, xbase, red, mkey, kbase, true, false);
+        }
         if (rotated)
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 sincos(va[i], &sn[i], &cs[i]);
@@ -437,7 +494,16 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
                 ef[nbus + i] = vm[i] * sn[i];
             }
         rotated = false;
-        return cl_mismatch<C>(a, rank, which, xbase, red, mkey, kbase, true, true);
+        return cl_mismatch<C>(a, rank, which, xbase, red, mkey, kbase, true);
+    };
+    auto half_mismatch = [&](int which) {
+        if (fx) {
+            const double m = cl_mismatch_fx<C>(a, rank, which, xbase, red, mkey, kbase, false, left);
+            if (__double_as_longlong(m) != -1ll) return m <= a.tol ? exact_check(which) : m;
+            enter_fp64();
+        }
+        const double m = cl_mismatch<C>(a, rank, which, xbase, red, mkey, kbase, false);
+        return m <= a.tol ? exact_check(which) : m;
     };
     // a step is followed by a cluster barrier (it read or feeds other CTAs'
     // words) or by the CTA's own barrier (a level of its own subtrees); every
@@ -458,8 +524,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
     };
     if (status == PF_ERR_NOT_CONVERGED) {
         for (int it = 0; it < a.max_iter; it++) {
-            mis = cl_mismatch<C>(a, rank, 0, xbase, red, mkey, kbase, false, true);
-            if (mis <= a.tol) mis = exact_check(0);
+            mis = half_mismatch(0);
             if (!isfinite(mis)) { status = PF_ERR_NONFINITE; break; }
             if (mis <= a.tol) { status = PF_OK; break; }
             solve(0);
@@ -467,6 +532,10 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
                 if (a.m[0].xref[i] < 0) continue;
                 const double d = xval(0, i);
                 va[i] += d;
+                if (fx) {
+                    left |= fx_angle_step(efx + i, d, vm[i], va[i]);
+                    continue;
+                }
                 if (fabs(d) <= kRotMax) {
                     double sd, cd;
                     small_sincos(d, &sd, &cd);
@@ -481,14 +550,18 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
             }
             rotated = true;
             iters++;
-            mis = cl_mismatch<C>(a, rank, 1, xbase, red, mkey, kbase, false, true);
-            if (mis <= a.tol) mis = exact_check(1);
+            mis = half_mismatch(1);
             if (!isfinite(mis)) { status = PF_ERR_NONFINITE; break; }
             if (mis <= a.tol) { status = PF_OK; break; }
             solve(1);
             for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
                 if (a.m[1].xref[i] < 0) continue;
-                vm[i] += xval(1, i);
+                const double d = xval(1, i);
+                vm[i] += d;
+                if (fx) {
+                    left |= fx_magnitude_step(efx + i, ivx + i, d, vm[i], va[i]);
+                    continue;
+                }
                 iv[i] = 1.0 / vm[i];
                 ef[i] = vm[i] * cs[i];
                 ef[nbus + i] = vm[i] * sn[i];
@@ -496,7 +569,8 @@ __global__ void __launch_bounds__(kClThreads, 1) k_fdpf_cl(const __grid_constant
             iters++;
         }
         if (status == PF_ERR_NOT_CONVERGED) {
-            mis = exact_check(0);
+            mis = half_mismatch(0);
+            if (!(mis <= a.tol)) mis = exact_check(0);
             if (mis <= a.tol) status = PF_OK;
         }
     }

