@@ -103,10 +103,69 @@ __global__ void __launch_bounds__(kTailInvWarps * 32) k_tail_inverse(const ClMat
     }
 }
 
+// The same column jt of a top too large for shared memory (and of a pack's
+// matrices): the columns of L_TT are read from L2, the next path node's range
+// and first entries while the current node is applied.
+template <class T>
+__device__ __forceinline__ void tail_inverse_column(const DevMat &m, const T *F, double *Wd, double *w, int jt) {
+    const int lane = threadIdx.x & 31, nt = m.nt;
+    for (int i = lane; i <= m.twdep[jt]; i += 32) w[i] = 0.0;
+    __syncwarp();
+    const int dj = m.twdep[jt];
+    if (lane == 0) w[0] = 1.0;
+    int a = m.twcp[jt], b = m.twcp[jt + 1], next = m.twpar[jt], dk = dj;
+    int ld = 0;
+    T lv = T(0);
+    if (a + lane < b) { ld = m.twcdep[a + lane]; lv = F[m.twcpos[a + lane]]; }
+    for (int k = jt; k >= 0;) {
+        const int ka = a, kb = b, kn = next, kd = ld, depk = dk;
+        const double kv = double(lv);
+        if (kn >= 0) {
+            a = m.twcp[kn];
+            b = m.twcp[kn + 1];
+            next = m.twpar[kn];
+            dk = m.twdep[kn];
+            if (a + lane < b) { ld = m.twcdep[a + lane]; lv = F[m.twcpos[a + lane]]; }
+        }
+        __syncwarp();
+        const double wk = w[dj - depk];
+        if (lane == 0) Wd[(long long)k * nt + jt] = wk;
+        if (ka + lane < kb) w[dj - kd] = fma(-kv, wk, w[dj - kd]);
+        for (int q = ka + lane + 32; q < kb; q += 32) {
+            const int pos = dj - m.twcdep[q];
+            w[pos] = fma(-double(F[m.twcpos[q]]), wk, w[pos]);
+        }
+        k = kn;
+    }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kTailInvWarps * 32) k_tail_inverse_l2(const DevMat m, const T *F, double *Wd) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    const int warp = threadIdx.x >> 5, jt = blockIdx.x * kTailInvWarps + warp;
+    if (jt < m.nt) tail_inverse_column<T>(m, F, Wd, reinterpret_cast<double *>(tsm) + warp * m.tw_depmax, jt);
+}
+
+template <class T>
+__global__ void __launch_bounds__(kTailInvWarps * 32)
+    k_tail_inverse_jobs(const FactorJob *jobs, int njob, const int *first, int depth_max) {
+    extern __shared__ __align__(16) unsigned char tsm[];
+    int lo = 0, hi = njob;  // the job of this block
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (first[mid] <= int(blockIdx.x)) lo = mid;
+        else hi = mid;
+    }
+    const FactorJob &J = jobs[lo];
+    const int warp = threadIdx.x >> 5, jt = (int(blockIdx.x) - first[lo]) * kTailInvWarps + warp;
+    if (jt < J.m.nt && J.m.npf3 > 0)
+        tail_inverse_column<T>(J.m, static_cast<const T *>(J.F), J.Wd, reinterpret_cast<double *>(tsm) + warp * depth_max, jt);
+}
+
 // Tail-inverse values of instance 0 (tail form 3 of the block engine):
 // forward entries W(i, j), backward entries W(j, i) / D(j), from the dense W.
 template <class T>
-__global__ void k_tw_values(const DevMat m, const double *Wd, const T *F, T *TW) {
+__device__ __forceinline__ void tw_values(const DevMat &m, const double *Wd, const T *F, T *TW) {
     const int tot = m.tw_nfe + m.tw_nbe;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += gridDim.x * blockDim.x) {
         if (e < m.tw_nfe) {
@@ -116,6 +175,17 @@ __global__ void k_tw_values(const DevMat m, const double *Wd, const T *F, T *TW)
             TW[m.tw_boff + b] = T(Wd[m.twbs[b]] * double(F[m.offDi + m.twbd[b]]));
         }
     }
+}
+
+template <class T>
+__global__ void k_tw_values(const DevMat m, const double *Wd, const T *F, T *TW) {
+    tw_values<T>(m, Wd, F, TW);
+}
+
+template <class T>
+__global__ void k_tw_values_jobs(const FactorJob *jobs) {
+    const FactorJob &J = jobs[blockIdx.y];
+    if (J.m.npf3 > 0 && J.TW) tw_values<T>(J.m, J.Wd, static_cast<const T *>(J.F), static_cast<T *>(J.TW));
 }
 
 // Packed values of the CTAs' programs (blockIdx.y = matrix): per slot
@@ -615,6 +685,17 @@ cudaError_t launch_tail_w(const DevMat &m, int prec, const void *F, double *Wd, 
     const int tot = m.tw_nfe + m.tw_nbe;
     const int vb = (tot + 255) / 256 < 1024 ? (tot + 255) / 256 : 1024;
     cudaError_t e;
+    if (smem > kTailInvSmem) {
+        const size_t sm2 = sizeof(double) * size_t(kTailInvWarps) * size_t(m.tw_depmax);
+        if (prec == PF_FP64) {
+            k_tail_inverse_l2<double><<<grid, kTailInvWarps * 32, sm2, s>>>(m, static_cast<const double *>(F), Wd);
+            k_tw_values<double><<<vb, 256, 0, s>>>(m, Wd, static_cast<const double *>(F), static_cast<double *>(TW));
+        } else {
+            k_tail_inverse_l2<float><<<grid, kTailInvWarps * 32, sm2, s>>>(m, static_cast<const float *>(F), Wd);
+            k_tw_values<float><<<vb, 256, 0, s>>>(m, Wd, static_cast<const float *>(F), static_cast<float *>(TW));
+        }
+        return cudaGetLastError();
+    }
     if (prec == PF_FP64) {
         e = cudaFuncSetAttribute(k_tail_inverse<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
@@ -625,6 +706,20 @@ cudaError_t launch_tail_w(const DevMat &m, int prec, const void *F, double *Wd, 
         if (e != cudaSuccess) return e;
         k_tail_inverse<float><<<grid, kTailInvWarps * 32, smem, s>>>(t, static_cast<const float *>(F), Wd);
         k_tw_values<float><<<vb, 256, 0, s>>>(m, Wd, static_cast<const float *>(F), static_cast<float *>(TW));
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tail_w_jobs(const FactorJob *jobs_dev, int njob, const int *first_dev, int nblocks, int depth_max,
+                               int prec, cudaStream_t s) {
+    if (nblocks == 0) return cudaSuccess;
+    const size_t smem = sizeof(double) * size_t(kTailInvWarps) * size_t(depth_max);
+    if (prec == PF_FP64) {
+        k_tail_inverse_jobs<double><<<nblocks, kTailInvWarps * 32, smem, s>>>(jobs_dev, njob, first_dev, depth_max);
+        k_tw_values_jobs<double><<<dim3(16, unsigned(njob)), 256, 0, s>>>(jobs_dev);
+    } else {
+        k_tail_inverse_jobs<float><<<nblocks, kTailInvWarps * 32, smem, s>>>(jobs_dev, njob, first_dev, depth_max);
+        k_tw_values_jobs<float><<<dim3(16, unsigned(njob)), 256, 0, s>>>(jobs_dev);
     }
     return cudaGetLastError();
 }

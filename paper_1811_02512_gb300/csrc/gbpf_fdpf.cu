@@ -2,8 +2,49 @@
 // (gbpf_fdpf.cuh; the kernels themselves are instantiated per precision in
 // gbpf_fdpf64.cu and gbpf_fdpf32.cu).
 #include "gbpf_fdpf.cuh"
+#include "gbpf_multi.cuh"
 
 namespace gbpf {
+
+namespace {
+// The sliced rows of a MultiNet from the current admittance matrix, a thread
+// per position: the fixed-point admittances, and with `refine` the rows of B'
+// and B'' (entries joining two of the matrix's buses) in units that take the
+// row's sum of magnitudes to at most 2^58.
+__global__ void k_multi_rows(DevNet dn, MultiNet N, int refine, double tol) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= dn.nbus) return;
+    const int2 ch = N.esl[p >> 5];
+    const int sl = p & 31, unit = N.meta[p].z + 2;  // the mismatch's units
+    N.tol[p] = fx_fits(tol, unit) ? fx_from_double(tol, unit) : 1ll << 62;
+    for (int c = ch.x; c < ch.x + ch.y; c++)
+        for (int u = 0; u < 4; u++) {
+            const int q = N.esrc[(4 * c + u) * 32 + sl];
+            N.eY[(4 * c + u) * 32 + sl] = q >= 0 ? dn.Yx[q] : make_int4(0, 0, 0, 0);
+        }
+    if (!refine) return;
+    for (int w = 0; w < 2; w++) {
+        auto value = [&](int c, int u) {
+            const int q = N.esrc[(4 * c + u) * 32 + sl];
+            const int4 col = N.ecol[c * 32 + sl];
+            const int o = u == 0 ? col.x : u == 1 ? col.y : u == 2 ? col.z : col.w;
+            if (q < 0 || N.row[w][p] < 0 || N.row[w][o] < 0) return 0.0;
+            return w == 0 ? dn.Bp[q] : -dn.B[q];
+        };
+        double l1 = 0.0;
+        for (int c = ch.x; c < ch.x + ch.y; c++)
+            for (int u = 0; u < 4; u++) l1 += fabs(value(c, u));
+        const int ex = int((unsigned(__double2hiint(l1)) >> 20) & 0x7ffu) - 1022;  // l1 < 2^ex
+        const int sc = kFxRow - min(max(ex, -400), 400);
+        N.qA[w][p] = make_int2(sc + 3, sc + 3 - unit);
+        for (int c = ch.x; c < ch.x + ch.y; c++)
+            for (int u = 0; u < 4; u++) {
+                const FxLimbs v = fx_split(fx_from_double(value(c, u), sc));
+                N.eA[w][(4 * c + u) * 32 + sl] = make_int2(v.h, v.l);
+            }
+    }
+}
+}  // namespace
 
 // ------------------------------------------------------------ launchers
 
@@ -54,12 +95,16 @@ void fill_run_args(RunArgs &a, const DevNet &dn, const DevCases &dc, const DevMa
     a.res = res;
     a.use_smem = 0;
     a.fallback = 0;
+    a.redo = nullptr;
 }
 
 size_t run_args_bytes() { return sizeof(RunArgs); }
 
+size_t fill_multi_args(MultiArgs &ma, const RunArgs &a, const MultiLaunch &ml, const DevMat *m, const void *Z0,
+                       const void *Z1, const double *K0, const double *K1, int prec);
+
 cudaError_t launch_pack(const PackGrid *grids, int ngrid, int prec, const pf_run_opts &o,
-                        const int *order_host, void *args_dev, int *order_dev, unsigned *counter_dev,
+                        const int *order_host, void *args_dev, void *margs_dev, int *order_dev, unsigned *counter_dev,
                         size_t smem_optin, int nsm, cudaStream_t s) {
     // the launch reserves shared memory for the largest grid whose solve
     // vector fits; larger grids keep theirs in global scratch
@@ -77,16 +122,79 @@ cudaError_t launch_pack(const PackGrid *grids, int ngrid, int prec, const pf_run
                       p.vm, p.va, p.ef, p.iv, p.xg, p.bmax, p.res);
         const int nm = p.m[0].n > p.m[1].n ? p.m[0].n : p.m[1].n;
         A[g].use_smem = nm <= ns;
+        A[g].TW0 = p.m[0].npf3 > 0 && A[g].TV0 ? p.TW0 : nullptr;
+        A[g].TW1 = p.m[1].npf3 > 0 && A[g].TV1 ? p.TW1 : nullptr;
+    }
+    // the several-cases-per-block kernel, one grid per block, takes every grid
+    // it fits; k_fdpf_pack below the others and what it left
+    std::vector<MultiArgs> M(static_cast<size_t>(ngrid));
+    size_t msmem = 0;
+    bool any = false;
+    for (int g = 0; g < ngrid; g++) {
+        const PackGrid &p = grids[g];
+        M[g].K = 0;
+        if (p.ml.K > 0) {
+            const size_t need = fill_multi_args(M[g], A[g], p.ml, p.m, nullptr, nullptr, nullptr, nullptr, prec);
+            if (need + sizeof(MultiArgs) + 1024 > smem_optin) {
+                M[g].K = 0;
+            } else {
+                msmem = need > msmem ? need : msmem;
+                any = true;
+                A[g].redo = p.ml.redo;
+                k_multi_rows<<<(p.dn.nbus + 127) / 128, 128, 0, s>>>(p.dn, p.ml.net, prec == PF_FP32 && o.ir_max > 0, o.tol);
+            }
+        }
+        A[g].TW0 = A[g].TW1 = nullptr;
     }
     cudaError_t e = cudaMemcpyAsync(args_dev, A.data(), sizeof(RunArgs) * size_t(ngrid),
                                     cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(order_dev, order_host, sizeof(int) * size_t(ngrid), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // A is released on return
+    if (e == cudaSuccess && any)
+        e = cudaMemcpyAsync(margs_dev, M.data(), sizeof(MultiArgs) * size_t(ngrid), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // A and M are released on return
     if (e != cudaSuccess) return e;
+    if (any) {
+        e = cudaMemsetAsync(counter_dev, 0, sizeof(unsigned), s);
+        if (e != cudaSuccess) return e;
+        const int blocks = ngrid < nsm ? ngrid : nsm;
+        const MultiArgs *ma = static_cast<const MultiArgs *>(margs_dev);
+        e = prec == PF_FP64 ? multi_pack_f64(ma, order_dev, ngrid, counter_dev, msmem, blocks, s)
+                            : multi_pack_f32(ma, order_dev, ngrid, counter_dev, msmem, blocks, s);
+        if (e != cudaSuccess) return e;
+    }
     return launch_fdpf_pack(static_cast<const RunArgs *>(args_dev), order_dev, ngrid, counter_dev, prec,
                             ring + elt * size_t(ns), nsm, s);
 }
+
+// The arguments of the several-cases-per-block kernel from those of k_fdpf;
+// returns its dynamic shared memory.
+size_t fill_multi_args(MultiArgs &ma, const RunArgs &a, const MultiLaunch &ml, const DevMat *m, const void *Z0,
+                       const void *Z1, const double *K0, const double *K1, int prec) {
+    const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
+    const int nmax = m[0].n > m[1].n ? m[0].n : m[1].n, nt = m[0].nt > m[1].nt ? m[0].nt : m[1].nt;
+    ma.r = a;
+    ma.K = ml.K;
+    ma.redo = ml.redo;
+    ma.net = ml.net;
+    ma.x = ml.x;
+    ma.xg = ml.xg;
+    for (int w = 0; w < 2; w++) {
+        ma.steps[w] = ml.steps[w];
+        ma.m[w] = m[w];
+        ma.F[w] = w == 0 ? a.F0 : a.F1;
+        ma.TV[w] = w == 0 ? a.TV0 : a.TV1;
+        ma.TW[w] = w == 0 ? a.TW0 : a.TW1;
+        ma.Z[w] = w == 0 ? Z0 : Z1;
+        ma.Kq[w] = w == 0 ? K0 : K1;
+        ma.xs0[w] = m[w].n > nmax - ml.xs0 ? m[w].n - (nmax - ml.xs0) : 0;
+    }
+    ma.zoff = ((nmax - ml.xs0) * ma.K + 3) & ~3;  // 16-byte accesses
+    ma.soff = int((elt * (size_t(ma.zoff) + size_t(nt) * size_t(ma.K)) + 15) & ~size_t(15));
+    return size_t(ma.soff) + sizeof(int2) * size_t(ma.steps[0].n() + ma.steps[1].n());
+}
+
+size_t multi_args_bytes() { return sizeof(MultiArgs); }
 
 // Cluster size of the power-flow kernel: a case spreads its nodal work over
 // 16 (or 8) SMs when the batch is too small to fill the GPU with one block per
@@ -110,8 +218,9 @@ cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, i
                         double *xg, double *bmax, pf_case_result *res, size_t smem_optin,
                         size_t smem_per_sm, int cluster, int threads, cudaStream_t s, const void *Z0,
                         const void *Z1, const double *K0, const double *K1, const NrLaunch *fb,
-                        const void *TW0, const void *TW1) {
+                        const void *TW0, const void *TW1, const int *redo, const MultiLaunch *multi) {
     RunArgs a;
+    a.redo = redo;
     a.Z0 = Z0;
     a.Z1 = Z1;
     a.K0 = K0;
@@ -168,8 +277,43 @@ cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, i
             a.fallback = 1;
         }
     }
+    if (multi && multi->K > 0) {
+        // several cases per block first; the launch below takes what it left
+        MultiArgs ma;
+        const size_t ms = fill_multi_args(ma, a, *multi, m, Z0, Z1, K0, K1, prec);
+        if (ms + 1024 > smem_optin) return cudaErrorInvalidConfiguration;
+        k_multi_rows<<<(dn.nbus + 127) / 128, 128, 0, s>>>(dn, ma.net, prec == PF_FP32 && o.ir_max > 0, o.tol);
+        const cudaError_t e = prec == PF_FP64 ? multi_run_f64(ma, ms, s) : multi_run_f32(ma, ms, s);
+        if (e != cudaSuccess) return e;
+        a.redo = multi->redo;
+    }
     return prec == PF_FP64 ? fdpf_run_f64(a, smem, cluster, threads, s)
                            : fdpf_run_f32(a, smem, cluster, threads, s);
+}
+
+int multi_cases(const DevMat *m, int prec, int ncase, int num_sms, size_t smem_optin, int *xs0) {
+    const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
+    const int nmax = m[0].n > m[1].n ? m[0].n : m[1].n;
+    const int nt = m[0].nt > m[1].nt ? m[0].nt : m[1].nt;
+    *xs0 = 0;
+    constexpr int kMultiStepBytes = 8192;  // the sweeps' steps (a few levels' and blocks' worth per matrix)
+    if (smem_optin < 32768) return 0;
+    // elements of the solve vectors and the top's vector that fit
+    const long long cap = (long long)((smem_optin - 2048 - kMultiStepBytes) / elt) - 4;
+    if (nmax + nt > cap) {
+        // one case, with rows below the narrow top (and at most half of
+        // them all) in global memory
+        const long long x = nmax + nt - cap;
+        if (x > m[0].n - m[0].nt || x > m[1].n || 2 * x > nmax) return 0;
+        *xs0 = int(x);
+        return 1;
+    }
+    int K = 0;
+    for (int k = 1; k <= kMultiMax && (long long)(nmax + nt) * k <= cap; k *= 2) {
+        K = k;
+        if ((ncase + k - 1) / k <= num_sms) break;
+    }
+    return K;
 }
 
 }  // namespace gbpf

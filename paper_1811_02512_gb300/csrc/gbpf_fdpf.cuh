@@ -48,6 +48,9 @@ struct RunArgs {
     // same launch; its result then reports method PF_NR
     int fallback;
     NrArgs nr;
+    // after k_fdpf_multi (or null): per case 0 done, 1 to be run, 2 its
+    // fallback only
+    const int *redo;
 };
 
 
@@ -394,6 +397,13 @@ __global__ void __launch_bounds__(kRunThreads, C == 1 ? 2 : 1) k_fdpf(const __gr
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ double red[33];
     __shared__ Ring R;
+    const int c = int(blockIdx.x) / C, redo = a.redo ? a.redo[c] : 1;  // the same in a case's cluster
+    if (redo == 0) return;
+    if (redo == 2) {
+        ring_init(&R);
+        nr_fallback<T, C>(a.nr, c, C == 1 ? 0 : int(cluster_rank()), smem_raw, red, &R);
+        return;
+    }
     fdpf_case<T, C>(a, int(blockIdx.x) / C, smem_raw, red, R, true);
 }
 
@@ -423,6 +433,7 @@ __global__ void __launch_bounds__(kRunThreads, 1)
         const bool broken = R.err != 0;
         __syncthreads();
         if (g < 0) break;
+        if (args[g].redo && args[g].redo[0] == 0) continue;  // done by k_fdpf_multi_pack
         if (broken) {
             if (threadIdx.x == 0) {
                 args[g].res[0].status = PF_ERR_TIMEOUT;

@@ -216,7 +216,8 @@ void build_tail_inverse(HostMat &H) {
         H.twcp[it + 1] = int(H.twcdep.size());
     }
     H.tw_ne = int(H.twcdep.size());
-    if (tail_inverse_smem(nt, H.tw_ne, depmax) > kTailInvSmem) return clear();
+    // the path values of k_tail_inverse_l2 within the default shared memory
+    if (sizeof(double) * size_t(kTailInvWarps) * size_t(depmax) > 48 * 1024) return clear();
     H.twpar = par;
     H.twdep = dep;
     H.tw_depmax = depmax;
@@ -522,20 +523,23 @@ pf_status build_tail(pf_ctx *ctx, HostMat &H, MakePieces &make_pieces, RunEnds &
     return PF_OK;
 }
 
-// Where the block factor changes from a warp per column to a warp per target
+// Where a factor changes from a warp per column to a warp per target
 // (see DevMat): the level above which the level-by-level form is the faster
 // one by the estimates below, in microseconds as measured on GB300.  By
 // columns a level costs its heaviest column (about 3, and 0.03 per update
 // term: the terms of a column run on one warp) per round of columns; by
 // targets a barrier and one pass of 32 terms per lane group and round of
-// targets (about 1, 1.5 and 0.6).  On a 20,000-bus grid the columns of the
-// narrow top carry thousands of terms each, all on one warp: the Newton
-// launch of four steps took 114 ms with a warp per column throughout.
+// targets (about 1, 1.5 and 0.6); for the scalar factor 2 and 0.01 against 1,
+// 1 and 0.4.  On a 20,000-bus grid the columns of the narrow top carry
+// thousands of terms each, all on one warp: the Newton launch of four steps
+// took 114 ms with a warp per column throughout.
 void split_block_factor(HostMat &H) {
     H.jlt.assign(H.nlev + 1, 0);
     for (int l = 0; l <= H.nlev; l++) H.jlt[l] = H.Cp[H.lvl_ptr[l]] + H.lvl_ptr[l];
-    const int warps[2] = {kSweepWarps, kSweepWarps * kClCtas};
-    for (int w = 0; w < 2; w++) {
+    const int warps[3] = {kSweepWarps, kSweepWarps * kClCtas, kSweepWarps * kClCtas};
+    const double cost[3][5] = {{3.0, 0.03, 1.0, 1.5, 0.6}, {3.0, 0.03, 1.0, 1.5, 0.6}, {2.0, 0.01, 1.0, 1.0, 0.4}};
+    for (int w = 0; w < 3; w++) {
+        const double *k = cost[w];
         H.jl0[w] = H.nlev;
         double gain = 0.0, best = 0.0;
         for (int l = H.nlev - 1; l >= 0; l--) {
@@ -546,8 +550,8 @@ void split_block_factor(HostMat &H) {
                 for (int t = t0; t < t1; t++) longest = std::max(longest, H.gp[t + 1] - H.gp[t]);
             }
             auto rounds = [](int n, int by) { return double((n + by - 1) / by); };
-            const double by_col = rounds(H.lvl_ptr[l + 1] - H.lvl_ptr[l], warps[w]) * (3.0 + 0.03 * heavy);
-            const double by_tgt = 1.0 + rounds(H.jlt[l + 1] - H.jlt[l], warps[w]) * (1.5 + 0.6 * rounds(longest, 32));
+            const double by_col = rounds(H.lvl_ptr[l + 1] - H.lvl_ptr[l], warps[w]) * (k[0] + k[1] * heavy);
+            const double by_tgt = k[2] + rounds(H.jlt[l + 1] - H.jlt[l], warps[w]) * (k[3] + k[4] * rounds(longest, 32));
             gain += by_col - by_tgt;
             if (gain > best) {
                 best = gain;
@@ -556,7 +560,7 @@ void split_block_factor(HostMat &H) {
         }
         H.jct[w] = H.lvl_ptr[H.jl0[w]];
     }
-    const int c0 = std::min(H.jct[0], H.jct[1]);
+    const int c0 = std::min(std::min(H.jct[0], H.jct[1]), H.jct[2]);
     H.jg0 = H.Cp[c0] + c0;
     H.jtcol.clear();
     for (int c = c0; c < H.n; c++) {
@@ -1419,7 +1423,7 @@ pf_status upload_matrix(pf_ctx *ctx, const HostMat &H, DevMat &D) {
     TRY(upload_padded(ctx, &D.jlt, H.jlt));
     TRY(upload_padded(ctx, &D.jtcol, H.jtcol));
     D.jg0 = H.jg0;
-    for (int w = 0; w < 2; w++) {
+    for (int w = 0; w < 3; w++) {
         D.jl0[w] = H.jl0[w];
         D.jct[w] = H.jct[w];
     }
@@ -1431,6 +1435,7 @@ pf_status upload_matrix(pf_ctx *ctx, const HostMat &H, DevMat &D) {
     D.t0 = H.t0;
     D.nt = H.nt;
     D.ntl = H.ntl;
+    TRY(upload_padded(ctx, &D.trange, std::vector<int>{H.t0, H.n}));
     D.npf2 = int(H.pf2.size());
     D.npb2 = int(H.pb2.size());
     D.npf3 = D.npb3 = 0;
@@ -1441,6 +1446,14 @@ pf_status upload_matrix(pf_ctx *ctx, const HostMat &H, DevMat &D) {
         TRY(upload(ctx, &D.twbc, H.twbc.data(), H.twbc.size()));
         TRY(upload_padded(ctx, &D.twfr, H.twfr));
         TRY(upload_padded(ctx, &D.twbr, H.twbr));
+        auto ends = [&](const std::vector<int> &rows, const std::vector<int2> &ch) {
+            std::vector<int> e(1, 0);  // entry ranges: the chunks of the rows follow one another
+            for (size_t r = 0; r + 1 < rows.size(); r++)
+                e.push_back(rows[r] < rows[r + 1] ? ch[size_t(rows[r + 1]) - 1].y : e.back());
+            return e;
+        };
+        TRY(upload_padded(ctx, &D.twfe, ends(H.twfr, H.twfc)));
+        TRY(upload_padded(ctx, &D.twbe, ends(H.twbr, H.twbc)));
         TRY(upload_padded(ctx, &D.twfj, H.twfj));
         TRY(upload_padded(ctx, &D.twbj, H.twbj));
         TRY(upload_padded(ctx, &D.twfs, H.twfs));
@@ -1713,6 +1726,9 @@ void free_case_storage(pf_ctx *ctx) {
     dfree(ctx, w.bmax); w.bmax = nullptr;
     dfree(ctx, w.iv); w.iv = nullptr;
     dfree(ctx, w.cstatus); w.cstatus = nullptr;
+    dfree(ctx, w.redo); w.redo = nullptr;
+    dfree(ctx, w.mx); w.mx = nullptr;
+    dfree(ctx, w.mxg); w.mxg = nullptr; w.mxg_count = 0;
     dfree(ctx, w.res); w.res = nullptr;
     dfree(ctx, ctx->dc.outage); ctx->dc.outage = nullptr;
     dfree(ctx, ctx->dc.inst); ctx->dc.inst = nullptr;
@@ -1764,13 +1780,16 @@ pf_status factor_job(pf_ctx *ctx, int which, int prec, FactorJob &J, cudaStream_
     J.done = w.fdone[which];
     J.amax = w.famax[which];
     J.epoch = w.fepoch[which];
+    J.Wd = w.TWd[which];
+    J.TW = w.TW[which][prec];
     return PF_OK;
 }
 
 // Assembles B' or B'' of every instance from the current admittance matrix
-// and factorises them.
+// and factorises them; top_inverse: with the partitioned inverse of the narrow
+// top of instance 0 (as tail form 3).
 pf_status factor_matrix(pf_ctx *ctx, int which, int prec, cudaStream_t s, int blocks_per_sm = 2,
-                        int ninst_f = -1) {
+                        int ninst_f = -1, bool top_inverse = false) {
     const int nf = ninst_f > 0 ? ninst_f : ctx->dc.ninst;  // instances factorised (the first nf)
     // only those are assembled: with low-rank outages the outage instances'
     // matrices are the base one minus the branch's share (U S U^T), which
@@ -1805,6 +1824,9 @@ pf_status factor_matrix(pf_ctx *ctx, int which, int prec, cudaStream_t s, int bl
     fs.tail = ctx->tune.tail != 2;
     fs.smem_optin = ctx->smem_optin;
     fs.partg = w.TP[which][prec];
+    // a top too large for the tail factor's shared memory: level by level
+    // through L2, by a cluster per instance
+    fs.top = nf <= 8 && fs.tail && factor_top_fits(prec);
     // the tail factor of a few instances on a cluster of SMs each
     fs.tail_cluster = false;
     if (m.ft_ng > 0 && nf <= 8 && nf * kTailCtas <= ctx->num_sms) {
@@ -1818,13 +1840,169 @@ pf_status factor_matrix(pf_ctx *ctx, int which, int prec, cudaStream_t s, int bl
     if (e != cudaSuccess) return cuda_fail(ctx, e, "factor launch");
     e = launch_tail_values(m, prec, F, w.TV[which][prec], nf, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "tail values launch");
-    if (ctx->tune.tail == 3 && m.npf3 > 0 && nf == 1) {
+    if ((ctx->tune.tail == 3 || top_inverse) && m.npf3 > 0 && nf == 1) {
         e = counted(ctx, PF_K_FACTOR, 2, s, [&] {
             return launch_tail_w(m, prec, F, w.TWd[which], w.TW[which][prec], s);
         });
         if (e != cudaSuccess) return cuda_fail(ctx, e, "tail inverse launch");
     }
     w.factored[which][prec] = true;
+    return PF_OK;
+}
+
+// Device tables of the several-cases-per-block kernel (see MultiNet).
+pf_status ensure_multi_net(pf_ctx *ctx) {
+    MultiNet &N = ctx->mnet;
+    if (N.qA[1]) return PF_OK;
+    const int nbus = ctx->nbus, nsl = (nbus + 31) / 32;
+    const std::vector<int> &rp = ctx->rowptr, &cl = ctx->col;
+    auto len = [&](int i) { return rp[i + 1] - rp[i]; };
+    // breadth-first order from a bus far from the slack, neighbours by degree
+    std::vector<int> ord, nb;
+    std::vector<char> seen;
+    auto bfs = [&](int root) {
+        ord.clear();
+        seen.assign(nbus, 0);
+        for (int s = -1; s < nbus; s++) {  // then whatever the pattern does not connect
+            const int r = s < 0 ? root : s;
+            if (seen[r]) continue;
+            seen[r] = 1;
+            size_t q = ord.size();
+            ord.push_back(r);
+            for (; q < ord.size(); q++) {
+                nb.clear();
+                for (int e = rp[ord[q]]; e < rp[ord[q] + 1]; e++)
+                    if (!seen[cl[e]]) {
+                        seen[cl[e]] = 1;
+                        nb.push_back(cl[e]);
+                    }
+                std::stable_sort(nb.begin(), nb.end(), [&](int a, int b) { return len(a) < len(b); });
+                ord.insert(ord.end(), nb.begin(), nb.end());
+            }
+        }
+    };
+    bfs(ctx->slack);
+    bfs(ord.back());
+    for (int p = 0; p < nbus; p += 1024)
+        std::stable_sort(ord.begin() + p, ord.begin() + std::min(nbus, p + 1024),
+                         [&](int a, int b) { return len(a) < len(b); });
+    std::vector<int> pos(nbus);
+    for (int p = 0; p < nbus; p++) pos[ord[p]] = p;
+    std::vector<int2> esl(nsl);
+    int nch = 0;
+    for (int s = 0; s < nsl; s++) {
+        int most = 1;
+        for (int p = 32 * s; p < std::min(nbus, 32 * s + 32); p++) most = std::max(most, len(ord[p]));
+        esl[s] = int2{nch, (most + 3) / 4};
+        nch += (most + 3) / 4;
+    }
+    std::vector<int4> ecol(size_t(nch) * 32, int4{0, 0, 0, 0}), meta(size_t(nsl) * 32, int4{0, 0, 0, 0});
+    std::vector<int> esrc(size_t(nch) * 128, -1), row[2];
+    for (int w = 0; w < 2; w++) row[w].assign(size_t(nsl) * 32, -1);
+    for (int p = 0; p < nbus; p++) {
+        const int i = ord[p], s = p / 32, l = p % 32;
+        meta[p] = int4{i, ctx->bus[i].type, ctx->ysc[i], 0};
+        for (int w = 0; w < 2; w++) row[w][p] = ctx->hm[w].new_of_bus[i];
+        for (int c = 0; c < esl[s].y; c++) {
+            int q[4];
+            for (int u = 0; u < 4; u++) {
+                const int e = ctx->rowptr[i] + 4 * c + u;
+                const bool in = e < ctx->rowptr[i + 1];
+                q[u] = in ? pos[ctx->col[e]] : p;
+                if (in) esrc[size_t(4 * (esl[s].x + c) + u) * 32 + l] = e;
+            }
+            ecol[size_t(esl[s].x + c) * 32 + l] = int4{q[0], q[1], q[2], q[3]};
+        }
+    }
+    N.nsl = nsl;
+    N.nchunk = nch;
+    TRY(upload(ctx, &N.esl, esl.data(), esl.size()));
+    TRY(upload(ctx, &N.ecol, ecol.data(), ecol.size()));
+    TRY(upload(ctx, &N.meta, meta.data(), meta.size()));
+    TRY(upload(ctx, &N.esrc, esrc.data(), esrc.size()));
+    TRY(upload(ctx, &N.pos, pos.data(), pos.size()));
+    TRY(dalloc(ctx, &N.eY, size_t(nch) * 128));
+    TRY(dalloc(ctx, &N.tol, size_t(nbus)));
+    for (int w = 0; w < 2; w++) {
+        TRY(upload(ctx, &N.row[w], row[w].data(), row[w].size()));
+        std::vector<int4> er(ecol.size());
+        for (size_t c = 0; c < ecol.size(); c++) {
+            const int q[4] = {ecol[c].x, ecol[c].y, ecol[c].z, ecol[c].w};
+            int v[4];
+            for (int u = 0; u < 4; u++) v[u] = std::max(0, row[w][q[u]]);
+            er[c] = int4{v[0], v[1], v[2], v[3]};
+        }
+        TRY(upload(ctx, &N.erow[w], er.data(), er.size()));
+        TRY(dalloc(ctx, &N.eA[w], size_t(nch) * 128));
+        TRY(dalloc(ctx, &N.qA[w], size_t(nsl) * 32));
+    }
+    return PF_OK;
+}
+
+// The steps of the sweeps of matrix `which` for `sub` lanes per row and entry
+// (see MultiSteps): a level's rows in blocks, with as many lanes per row as
+// fill the block and the rows' mean length asks for (FP64: two entries a
+// lane, as its additions across lanes cost as much as a product).  Levels
+// whose rows have no entries (the leaves, forward) are left out.
+pf_status ensure_multi_steps(pf_ctx *ctx, int which, int prec, int K, bool top, MultiSteps &out) {
+    const int sub = prec == PF_FP64 ? K : 1, lg = prec == PF_FP64 ? (K >= 4 ? 3 : K == 2 ? 2 : 1) : 0;
+    MultiSteps &S = ctx->msteps[which][lg][top];
+    const HostMat &H = ctx->hm[which];
+    if (!S.steps) {
+        std::vector<int2> v;
+        auto add = [&]( const std::vector<int> &ptr, int a, int b, bool diag) {
+            const int ne = ptr[b] - ptr[a], lanes = kMultiThreads / sub;
+            if (a >= b || (ne == 0 && !diag)) return;
+            int lg = 0;
+            while ((1 << lg) < 32 / sub && (b - a) * (2 << lg) <= lanes && (b - a) << lg < ne / (prec == PF_FP64 ? 2 : 1))
+                lg++;
+            const int per = lanes >> lg;
+            for (int r = a; r < b; r += per)
+                v.push_back(int2{r | int(unsigned(lg) << 28),
+                                 std::min(b - r, per) | int(r + per >= b ? 1u << 31 : 0u)});
+        };
+        const int lb = top ? H.nlev - H.ntl : H.nlev;
+        for (int l = 0; l < lb; l++) add(H.Fp, H.lvl_ptr[l], H.lvl_ptr[l + 1], false);
+        S.nf = int(v.size());
+        if (top) add(H.PPp, H.t0, H.n, true);
+        S.np = int(v.size()) - S.nf;
+        for (int l = lb - 1; l >= 0; l--) add(H.Cp, H.lvl_ptr[l], H.lvl_ptr[l + 1], true);
+        S.nb = int(v.size()) - S.nf - S.np;
+        if (v.empty()) v.push_back(int2{0, 0});
+        TRY(upload(ctx, &S.steps, v.data(), v.size()));
+    }
+    out = S;
+    return PF_OK;
+}
+
+// The several-cases-per-block launch of this batch: its shape and storage (K
+// = 0: it does not apply).
+pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, MultiLaunch &ml) {
+    Workspace &w = ctx->ws;
+    ml.K = multi_cases(ctx->dm, prec, ctx->dc.ncase, ctx->num_sms, ctx->smem_optin, &ml.xs0);
+    if (ml.K == 0) return PF_OK;
+    TRY(ensure_multi_net(ctx));
+    ml.net = ctx->mnet;
+    for (int q = 0; q < 2; q++)
+        TRY(ensure_multi_steps(ctx, q, prec, ml.K, ctx->dm[q].npf3 > 0, ml.steps[q]));
+    if (!w.redo) TRY(dalloc(ctx, &w.redo, size_t(ctx->dc.ncase)));
+    ml.redo = w.redo;
+    const size_t rows = size_t(ctx->dc.ncase) * size_t(ml.xs0);
+    if (rows > w.mxg_count) {
+        drop_graph(ctx);
+        dfree(ctx, w.mxg);
+        w.mxg = nullptr;
+        w.mxg_count = 0;
+        double *p = nullptr;
+        TRY(dalloc(ctx, &p, rows));
+        w.mxg = p;
+        w.mxg_count = rows;
+    }
+    ml.xg = w.mxg;
+    if (prec == PF_FP32 && refine) {
+        if (!w.mx) TRY(dalloc(ctx, &w.mx, size_t(ctx->dc.ncase) * size_t(ctx->nbus)));
+        ml.x = w.mx;
+    }
     return PF_OK;
 }
 
@@ -1870,7 +2048,8 @@ pf_status prepare_lowrank(pf_ctx *ctx, int prec, cudaStream_t s) {
 // instances) the two factorisations are independent chains of dependent
 // columns: B'' runs on a second stream beside B', each launch capped at one
 // block per SM so both are resident at once.
-pf_status factor_both(pf_ctx *ctx, int prec, cudaStream_t s, bool lowrank, bool cl_inverse = false) {
+pf_status factor_both(pf_ctx *ctx, int prec, cudaStream_t s, bool lowrank, bool cl_inverse = false,
+                      bool top_inverse = false) {
     Workspace &w = ctx->ws;
     const int ninst = lowrank ? 1 : ctx->dc.ninst;
     const bool dep = ctx->tune.factor == 1 || (ctx->tune.factor == 0 && ninst < ctx->num_sms / 2);
@@ -1885,9 +2064,9 @@ pf_status factor_both(pf_ctx *ctx, int prec, cudaStream_t s, bool lowrank, bool 
         return e == cudaSuccess ? PF_OK : cuda_fail(ctx, e, "top inverse");
     };
     if (!dep) {
-        TRY(factor_matrix(ctx, PF_MAT_BP, prec, s, 2, ninst));
+        TRY(factor_matrix(ctx, PF_MAT_BP, prec, s, 2, ninst, top_inverse));
         TRY(inverse(PF_MAT_BP, s));
-        TRY(factor_matrix(ctx, PF_MAT_BPP, prec, s, 2, ninst));
+        TRY(factor_matrix(ctx, PF_MAT_BPP, prec, s, 2, ninst, top_inverse));
         TRY(inverse(PF_MAT_BPP, s));
         return PF_OK;
     }
@@ -1900,9 +2079,9 @@ pf_status factor_both(pf_ctx *ctx, int prec, cudaStream_t s, bool lowrank, bool 
     cudaError_t e = cudaEventRecord(w.fork, s);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(w.side, w.fork, 0);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fork");
-    TRY(factor_matrix(ctx, PF_MAT_BPP, prec, w.side, 1, ninst));
+    TRY(factor_matrix(ctx, PF_MAT_BPP, prec, w.side, 1, ninst, top_inverse));
     TRY(inverse(PF_MAT_BPP, w.side));
-    TRY(factor_matrix(ctx, PF_MAT_BP, prec, s, 1, ninst));
+    TRY(factor_matrix(ctx, PF_MAT_BP, prec, s, 1, ninst, top_inverse));
     TRY(inverse(PF_MAT_BP, s));
     e = cudaEventRecord(w.join, w.side);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, w.join, 0);
@@ -2503,8 +2682,20 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
         if (e != cudaSuccess) return cuda_fail(ctx, e, "cluster fdpf launch");
         return PF_OK;
     }
+    // several cases per block, wherever all solves use the base factor and the
+    // tuning names no other tail form, block size or cluster: faster than
+    // k_fdpf at every size tried, a single case on one SM included, where
+    // k_fdpf's 16-block cluster shares only the nodal work (FP32, ir_tol 1e-3:
+    // 0.27 ms against 0.55 on 200 buses, 0.87 against 1.35 on 2,643, 7.4
+    // against 11.5 on 40,000; FP64 0.38 against 0.54, 11.1 against 14.6 on
+    // 40,000).
+    MultiLaunch ml;
+    const bool multi = (ctx->tune.tail == 0 || ctx->tune.tail == 3) &&
+                       (ctx->tune.threads == 0 || ctx->tune.threads == 512) && ctx->tune.cluster <= 1;
+    if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2))
+        TRY(ensure_multi(ctx, prec, opts->ir_max > 0, ml));
     const bool lowrank = ctx->tune.outage == 2 && ctx->dc.ninst > 1;
-    TRY(factor_both(ctx, prec, s, lowrank));
+    TRY(factor_both(ctx, prec, s, lowrank, false, ml.K > 0));
     if (lowrank) {
         TRY(prepare_lowrank(ctx, prec, s));
         // the outage instances' own factors were not computed: pf_solve and
@@ -2518,7 +2709,7 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     if (ctx->tune.cluster > 0 && ctx->tune.cluster < cl) cl = ctx->tune.cluster < 8 ? 1 : 8;
     const bool tail = ctx->tune.tail != 2;
     // tail form 3: every case's solves use the factor of instance 0
-    const bool tw = ctx->tune.tail == 3 && (ctx->dc.ninst == 1 || lowrank);
+    const bool tw = (ctx->tune.tail == 3 || ml.K > 0) && (ctx->dc.ninst == 1 || lowrank);
     cudaError_t e = counted(ctx, PF_K_RUN, 1, s, [&] {
         return launch_fdpf(ctx->dn, ctx->dc, ctx->dm, prec, F0, F1, tail ? w.TV[0][prec] : nullptr,
                            tail ? w.TV[1][prec] : nullptr, w.A[0], w.A[1], w.fstatus[0][prec],
@@ -2527,7 +2718,7 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
                            lowrank ? w.LZ[0][prec] : nullptr,
                            lowrank ? w.LZ[1][prec] : nullptr, lowrank ? w.LK[0] : nullptr,
                            lowrank ? w.LK[1] : nullptr, fb, tw ? w.TW[0][prec] : nullptr,
-                           tw ? w.TW[1][prec] : nullptr);
+                           tw ? w.TW[1][prec] : nullptr, nullptr, &ml);
     });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fdpf launch");
     return PF_OK;
@@ -2962,10 +3153,13 @@ struct pf_pack {
     std::vector<int> order;       // grids by decreasing size
     std::vector<int64_t> offset;  // first bus of each grid in the concatenated state
     std::vector<int2> items;      // factor work items (job = 2 grid + matrix, column)
+    size_t n_below = 0;           // the first of them: columns below their matrix's top levels (jct[2])
     int2 *items_dev = nullptr;
     gbpf::FactorJob *jobs_dev = nullptr;
     unsigned *fsync = nullptr;
-    void *args = nullptr;
+    void *args = nullptr, *margs = nullptr;
+    int *tw_first = nullptr;      // first block of every job's top inverse
+    int tw_blocks = 0, tw_depth = 0;
     int *order_dev = nullptr;
     unsigned *counter = nullptr;
     pf_case_result *res = nullptr;
@@ -3025,13 +3219,17 @@ pf_status pf_pack_create(pf_ctx *const *grids, int32_t ngrid, pf_pack **out) {
     int maxlev = 0;
     for (pf_ctx *c : pk->grids)
         for (int w = 0; w < 2; w++) maxlev = std::max(maxlev, c->hm[w].nlev);
+    std::vector<int2> top;
     for (int l = 0; l < maxlev; l++)
         for (int g = 0; g < ngrid; g++)
             for (int w = 0; w < 2; w++) {
                 const gbpf::HostMat &H = pk->grids[g]->hm[w];
                 if (l >= H.nlev) continue;
-                for (int c = H.lvl_ptr[l]; c < H.lvl_ptr[l + 1]; c++) pk->items.push_back(int2{2 * g + w, c});
+                for (int c = H.lvl_ptr[l]; c < H.lvl_ptr[l + 1]; c++)
+                    (c < H.jct[2] ? pk->items : top).push_back(int2{2 * g + w, c});
             }
+    pk->n_below = pk->items.size();
+    pk->items.insert(pk->items.end(), top.begin(), top.end());
     *out = pk;
     return PF_OK;
 }
@@ -3070,6 +3268,12 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
         p.F1 = prec == PF_FP64 ? (const void *)w.F64[1] : (const void *)w.F32[1];
         p.TV0 = ctx->tune.tail != 2 ? w.TV[0][prec] : nullptr;
         p.TV1 = ctx->tune.tail != 2 ? w.TV[1][prec] : nullptr;
+        p.TW0 = w.TW[0][prec];
+        p.TW1 = w.TW[1][prec];
+        if (ctx->tune.tail == 0 || ctx->tune.tail == 3) {
+            st = ensure_multi(ctx, prec, opts->ir_max > 0, p.ml);
+            if (st != PF_OK) return pack_fail(pk, st, "grid %d: %s", g, ctx->err.c_str());
+        }
         p.A0 = w.A[0];
         p.A1 = w.A[1];
         p.fs0 = w.fstatus[0][prec];
@@ -3097,6 +3301,18 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
             e = cudaMalloc(reinterpret_cast<void **>(&pk->items_dev), sizeof(int2) * std::max<size_t>(1, pk->items.size()));
         if (e == cudaSuccess)
             e = cudaMemcpy(pk->items_dev, pk->items.data(), sizeof(int2) * pk->items.size(), cudaMemcpyHostToDevice);
+        std::vector<int> first(1, 0);  // blocks of the tops' inverses per job
+        for (pf_ctx *ctx : pk->grids)
+            for (int w = 0; w < 2; w++) {
+                const DevMat &m = ctx->dm[w];
+                first.push_back(first.back() + (m.npf3 > 0 ? (m.nt + gbpf::kTailInvWarps - 1) / gbpf::kTailInvWarps : 0));
+                pk->tw_depth = std::max(pk->tw_depth, m.npf3 > 0 ? m.tw_depmax : 0);
+            }
+        pk->tw_blocks = first.back();
+        if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&pk->tw_first), sizeof(int) * first.size());
+        if (e == cudaSuccess)
+            e = cudaMemcpy(pk->tw_first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMalloc(&pk->margs, multi_args_bytes() * size_t(ngrid));
         if (e == cudaSuccess) e = cudaMalloc(&pk->args, run_args_bytes() * size_t(ngrid));
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&pk->order_dev), sizeof(int) * size_t(ngrid));
         if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void **>(&pk->counter), sizeof(unsigned));
@@ -3109,15 +3325,18 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
     // every grid's B' and B'' in one factor launch
     e = cudaMemcpyAsync(pk->jobs_dev, jobs.data(), sizeof(FactorJob) * jobs.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);  // jobs is released on return
+    const bool top = factor_top_fits(prec);
     if (e == cudaSuccess)
-        e = launch_factor_jobs(pk->jobs_dev, 2 * ngrid, pk->items_dev, unsigned(pk->items.size()), pk->fsync,
-                               prec, pk->num_sms, s);
+        e = launch_factor_jobs(pk->jobs_dev, 2 * ngrid, pk->items_dev,
+                               unsigned(top ? pk->n_below : pk->items.size()), pk->fsync, prec, pk->num_sms, top, s);
+    if (e == cudaSuccess)
+        e = launch_tail_w_jobs(pk->jobs_dev, 2 * ngrid, pk->tw_first, pk->tw_blocks, pk->tw_depth, prec, s);
     if (e != cudaSuccess)
         return pack_fail(pk, e == cudaErrorMemoryAllocation ? PF_ERR_OOM : PF_ERR_CUDA, "pack factor: %s",
                          cudaGetErrorString(e));
     for (pf_ctx *ctx : pk->grids)
         for (int w = 0; w < 2; w++) ctx->ws.factored[w][prec] = true;
-    e = launch_pack(pg.data(), ngrid, prec, *opts, pk->order.data(), pk->args, pk->order_dev, pk->counter,
+    e = launch_pack(pg.data(), ngrid, prec, *opts, pk->order.data(), pk->args, pk->margs, pk->order_dev, pk->counter,
                     pk->smem_optin, pk->num_sms, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(res_host, pk->res, sizeof(pf_case_result) * size_t(ngrid), cudaMemcpyDeviceToHost, s);
@@ -3137,6 +3356,8 @@ const char *pf_pack_last_error(const pf_pack *pk) { return pk ? pk->err.c_str() 
 void pf_pack_destroy(pf_pack *pk) {
     if (!pk) return;
     cudaFree(pk->args);
+    cudaFree(pk->margs);
+    cudaFree(pk->tw_first);
     cudaFree(pk->jobs_dev);
     cudaFree(pk->items_dev);
     cudaFree(pk->fsync);

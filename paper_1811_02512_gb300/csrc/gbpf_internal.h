@@ -82,6 +82,7 @@ struct DevMat {
     // into [tv_f: forward slots | tv_b: backward slots | tv_p: entries below
     // t0] from the value slots TVsrc (-1: zero).
     int t0 = 0, nt = 0, ntl = 0;
+    int *trange = nullptr;     // {t0, n}
     int npf2 = 0, npb2 = 0;
     Piece *pf2 = nullptr, *pb2 = nullptr;
     int *SKf = nullptr, *SIf = nullptr, *SKb = nullptr, *SIb = nullptr;
@@ -132,6 +133,7 @@ struct DevMat {
     int tw_nfc = 0, tw_nbc = 0, tw_nfe = 0, tw_nbe = 0, tw_boff = 0, tw_stride = 0;
     int2 *twfc = nullptr, *twbc = nullptr;
     int *twfr = nullptr, *twbr = nullptr, *twfj = nullptr, *twbj = nullptr;
+    int *twfe = nullptr, *twbe = nullptr;  // [nt + 1] rows' entry ranges (their chunks joined)
     int *twfs = nullptr, *twbs = nullptr, *twbd = nullptr;
     int *twpar = nullptr, *twcp = nullptr, *twcdep = nullptr, *twcpos = nullptr, *twdep = nullptr;
     int tw_ne = 0, tw_depmax = 0;
@@ -141,12 +143,13 @@ struct DevMat {
     int npfJ = 0, npbJ = 0;
     Piece *pfJ = nullptr, *pbJ = nullptr;
     int *srcT = nullptr;       // [nnz] Ybus position of the transposed entry (c, r) of each slot
-    // Top levels of the block factor, factorised level by level with a warp
-    // per target: from level jl0[w] (first column jct[w]) up, w = 0 for the
-    // warps of one block per case, 1 for a cluster's.  jlt[l]: first target
+    // Top levels of a factor, factorised level by level with a warp per
+    // target: from level jl0[w] (first column jct[w]) up, w = 0 for the block
+    // factor by the warps of one block per case, 1 by a cluster's, 2 for the
+    // scalar factor by a cluster's (k_factor_top).  jlt[l]: first target
     // (Cp[c] + c of the level's first column) of level l, [nlev + 1]; jtcol:
     // column c of every target from jg0 on, ~c for a diagonal.
-    int jl0[2] = {0, 0}, jct[2] = {0, 0}, jg0 = 0;
+    int jl0[3] = {0, 0, 0}, jct[3] = {0, 0, 0}, jg0 = 0;
     int *jlt = nullptr, *jtcol = nullptr;
     int jD = 0, jDi = 0, jLc = 0, jUc = 0, jLr = 0, jUr = 0, jstride = 0;  // block layout (elements)
 };
@@ -267,7 +270,7 @@ struct HostMat {
     std::vector<int> Ap, Aj, Apos;    // off-diagonal pattern of A by row (both triangles, no fill)
     std::vector<Piece> pfJ, pbJ;
     std::vector<int> srcT;
-    int jl0[2] = {0, 0}, jct[2] = {0, 0}, jg0 = 0;
+    int jl0[3] = {0, 0, 0}, jct[3] = {0, 0, 0}, jg0 = 0;
     std::vector<int> jlt, jtcol;
     int jD = 0, jDi = 0, jLc = 0, jUc = 0, jLr = 0, jUr = 0, jstride = 0;
     std::vector<Piece> pf, pb;
@@ -362,6 +365,53 @@ struct LaneSet {
     int prec = -1;
 };
 
+// Several cases per block (gbpf_multi.cuh): K cases, their marks for the
+// k_fdpf launch that follows, and for FP32 the refined solutions and the
+// fixed-point rows of B' and B'' (formed by the launch from A).
+//
+// Its network tables are in position order: position p is bus meta[p].x.
+// Positions follow a breadth-first (Cuthill-McKee) numbering of the grid, so
+// that the neighbours a warp gathers lie close together and stay in the L1,
+// sorted by row length within windows of 1,024.  The rows of the
+// admittance matrix are stored by slices of 32 positions in chunks of four
+// entries, so that a warp's loads are contiguous: slice s has chunks [esl[s].x,
+// esl[s].x + esl[s].y); chunk c of position p holds the neighbours' positions
+// ecol[32 c + p % 32] and entry u at index 32 (4 c + u) + p % 32 of eY (limbs
+// in the row's units), of eA[w] (B' and B'' on the same pattern) and of esrc
+// (the Ybus position, -1 padding).  qA[w][p]: {q, shift}: the row's sums of
+// eA times a solution in units 2^-60 are in units 2^-q, a right-hand side in
+// the bus's units comes to them by a left shift (tol: the run's tolerance in
+// the bus's units).
+struct MultiNet {
+    int nsl = 0, nchunk = 0;
+    int2 *esl = nullptr;
+    int4 *ecol = nullptr, *eY = nullptr, *meta = nullptr;  // meta: {bus, type, ysc, 0}
+    int *esrc = nullptr, *pos = nullptr;                   // pos: position of a bus
+    int *row[2] = {nullptr, nullptr};                      // B', B'' row of a position, -1
+    int2 *eA[2] = {nullptr, nullptr};
+    int4 *erow[2] = {nullptr, nullptr};                    // ecol as rows of B', B'' (0: absent)
+    int2 *qA[2] = {nullptr, nullptr};
+    long long *tol = nullptr;
+};
+constexpr int kMultiThreads = 512;  // threads of a block
+// Steps of the kernel's sweeps of one matrix: forward below the top, the top
+// rows' entries below it (none: no inverse of the top), backward, one after
+// the other; {first row | log2 lanes per row << 28, rows | 1 << 31 where a
+// barrier follows}.
+struct MultiSteps {
+    int nf = 0, np = 0, nb = 0;
+    int2 *steps = nullptr;
+    __host__ __device__ int n() const { return nf + np + nb; }
+};
+struct MultiLaunch {
+    int K = 0;
+    int xs0 = 0;               // rows of the solve vector kept in global memory
+    int *redo = nullptr;       // [ncase]
+    int2 *x = nullptr;         // [ncase][nbus]
+    void *xg = nullptr;        // [ncase][xs0] of the factor type
+    MultiSteps steps[2];
+    MultiNet net;
+};
 struct FactorJob;
 
 struct Workspace {
@@ -397,6 +447,10 @@ struct Workspace {
     double *bmax = nullptr;   // [ncase][16] per-CTA mismatch maxima and solve flag
     double *iv = nullptr;     // [ncase][nbus] 1 / V
     int *cstatus = nullptr;   // [ncase] run status
+    int *redo = nullptr;      // [ncase] marks of k_fdpf_multi
+    int2 *mx = nullptr;       // [ncase][nbus] its refined solutions (FP32)
+    void *mxg = nullptr;      // [ncase][rows in global memory] of 8 bytes
+    size_t mxg_count = 0;
     pf_case_result *res = nullptr; // [ncase]
     int ncase_alloc = 0;
     double *lsbuf = nullptr;  // [ncase][nbus] load scales of the batch (kept for a cheap re-set)
@@ -438,6 +492,8 @@ struct pf_ctx {
     gbpf::HostMat hm[2];
     gbpf::DevMat dm[2];
     gbpf::DevNet dn;
+    gbpf::MultiNet mnet;  // tables of the several-cases-per-block kernel (on first use)
+    gbpf::MultiSteps msteps[2][4][2];  // [mat][FP32; FP64 by 1, 2, 4 cases][without, with the top's inverse]
     gbpf::DevCases dc;
     gbpf::Workspace ws;
     bool on_device = false;   // network and symbolic data uploaded
@@ -502,6 +558,7 @@ struct FactorSync {
     void *partg = nullptr;     // [ninst][ft_ng] of the factor type: the tail targets' parts
                                // from columns below the tail (k_factor_tail_pre)
     bool tail_cluster = false; // the tail factor of every instance on a cluster of kTailCtas CTAs
+    bool top = false;          // without the tail factor: the top levels by k_factor_top
 };
 constexpr int kTailCtas = 16;  // CTAs of the tail factor's cluster (one per SM)
 size_t factor_tail_smem(const DevMat &m, int prec);
@@ -521,15 +578,25 @@ struct FactorJob {
     unsigned *done;
     double *amax;
     unsigned epoch;
+    double *Wd;  // dense inverse of the narrow top, its gathered values (or null)
+    void *TW;
 };
 // Factorises the matrices jobs_dev[0..njob) in one dependency-driven launch
 // over the work items (job, column) of items_dev (every column after the
 // columns it depends on), then gathers their tail values.  sync_dev: the
 // column counter and abort flag.
+// top: the items are the columns below jct[2] of every matrix and the levels
+// above follow by k_factor_top.
 cudaError_t launch_factor_jobs(const FactorJob *jobs_dev, int njob, const int2 *items_dev,
-                               unsigned nitems, unsigned *sync_dev, int prec, int nsm, cudaStream_t s);
+                               unsigned nitems, unsigned *sync_dev, int prec, int nsm, bool top, cudaStream_t s);
+// Whether a cluster of k_factor_top can be resident.
+bool factor_top_fits(int prec);
 // Partitioned inverse of the narrow top of instance 0 (tail form 3): the
 // dense W = L_TT^-1 into Wd (FP64) and the gathered values into TW (prec).
+// The same for the matrices of a pack; first_dev: each job's first block of
+// kTailInvWarps columns, [njob + 1]; smem: the largest path's.
+cudaError_t launch_tail_w_jobs(const FactorJob *jobs_dev, int njob, const int *first_dev, int nblocks, int depth_max,
+                               int prec, cudaStream_t s);
 cudaError_t launch_tail_w(const DevMat &m, int prec, const void *F, double *Wd, void *TW, cudaStream_t s);
 cudaError_t launch_tail_values(const DevMat &m, int prec, const void *F, void *TV, int ninst,
                                cudaStream_t s);
@@ -545,6 +612,9 @@ cudaError_t launch_mismatch(const DevNet &dn, const DevCases &dc, const double *
                             double *dp, double *dq, double *maxmis, double *ef, int ncase,
                             cudaStream_t s);
 struct NrLaunch;
+// Cases per block for a batch: as few as let every block run at once, as
+// many as fit shared memory at most; 0 where not even one does.
+int multi_cases(const DevMat *m, int prec, int ncase, int num_sms, size_t smem_optin, int *xs0);
 // fb (optional): the Newton-Raphson launch that unconverged cases fall back
 // to inside the same launch (ignored when its factor scratch does not fit);
 // TW0/TW1 (optional): tail-inverse values of instance 0 (tail form 3).
@@ -557,7 +627,8 @@ cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, i
                         int threads, cudaStream_t s,
                         const void *Z0 = nullptr, const void *Z1 = nullptr, const double *K0 = nullptr,
                         const double *K1 = nullptr, const NrLaunch *fb = nullptr,
-                        const void *TW0 = nullptr, const void *TW1 = nullptr);
+                        const void *TW0 = nullptr, const void *TW1 = nullptr, const int *redo = nullptr,
+                        const MultiLaunch *multi = nullptr);
 // Z = A^-1 U and K = (I - S U^T Z)^-1 S of every outage instance of matrix
 // `which` from the base factor F (instance 0): the low-rank form of the
 // outage cases.  gvec: [2 (ninst - 1)][n] scratch of the factor type.
@@ -573,18 +644,20 @@ struct PackGrid {
     DevNet dn;
     DevCases dc;
     DevMat m[2];
-    const void *F0, *F1, *TV0, *TV1;
+    const void *F0, *F1, *TV0, *TV1, *TW0, *TW1;
     const double *A0, *A1;
     const int *fs0, *fs1;
     double *vm, *va, *ef, *iv, *xg, *bmax;
     pf_case_result *res;
+    MultiLaunch ml;
 };
 size_t run_args_bytes();
+size_t multi_args_bytes();
 // Runs every grid of a pack to tolerance in one persistent launch (grids
 // taken largest first, order_host); args_dev/order_dev/counter_dev are
 // device scratch of ngrid run arguments, ngrid ints and one counter.
 cudaError_t launch_pack(const PackGrid *grids, int ngrid, int prec, const pf_run_opts &o,
-                        const int *order_host, void *args_dev, int *order_dev, unsigned *counter_dev,
+                        const int *order_host, void *args_dev, void *margs_dev, int *order_dev, unsigned *counter_dev,
                         size_t smem_optin, int nsm, cudaStream_t s);
 
 // One launch of the Newton-Raphson kernel (adjoint = false) or of the

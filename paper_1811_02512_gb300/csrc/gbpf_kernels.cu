@@ -637,6 +637,105 @@ __global__ void __launch_bounds__(kDepThreads)
     }
 }
 
+// The top levels of the factor of one instance by a cluster (this CTA is
+// `rank` of C), after the columns below jct[2] are done: level by level with a
+// warp per target, in the form of block_factor_top (unnormalised entries
+// U_ic = L_ic D_c until the end, so a level needs no division pass),
+//   U_ic = A_ic - sum_k L_ik (M_k L_ck),  M_k = D_k below, 1/D_k in the top
+// (where the entries read are U).  For tops too large for the tail factor's
+// shared memory, and for packs: there the columns of the top carry thousands
+// of terms and took one warp each.  Bound by the latency of a level through
+// L2.
+template <class T, int C>
+__device__ void factor_top(const DevMat &mr, const double *a, T *v, int *fstat, double amax, int rank) {
+    const DevMat m = mr;
+    const int lane = threadIdx.x & 31, nw = int(blockDim.x >> 5);
+    const int gw = rank * nw + int(threadIdx.x >> 5), W = C * nw;
+    const int ct = m.jct[2], l0 = m.jl0[2];
+    T *Lc = v + m.offLc, *Di = v + m.offDi;
+    if (l0 >= m.nlev) return;
+    const int tend = m.jlt[m.nlev];
+    int lo = 0, hi = 0, col = 0;
+    int4 e0 = make_int4(0, 0, 0, 0), e1 = e0;
+    auto fetch = [&](int t) {  // a target and its first terms' indices
+        lo = m.gp[t];
+        hi = m.gp[t + 1];
+        col = m.jtcol[t - m.jg0];
+        if (lo + lane < hi) e0 = __ldg(m.gl + lo + lane);
+        if (lo + 32 + lane < hi) e1 = __ldg(m.gl + lo + 32 + lane);
+    };
+    int ta = m.jlt[l0], te = m.jlt[l0 + 1];
+    if (ta + gw < te) fetch(ta + gw);
+    for (int l = l0; l < m.nlev; l++) {
+        const int tn = l + 1 < m.nlev ? m.jlt[l + 2] : tend;
+        for (int t = ta + gw; t < te; t += W) {
+            if (t != ta + gw) fetch(t);
+            const bool diag = col < 0;
+            const int cc = diag ? ~col : col, p = t - cc - 1;
+            const double src = a[diag ? cc : m.offLc + p];
+            T s = T(0);
+            for (int g = lo; g < hi; g += 64) {  // two terms per lane in flight
+                const int g0 = g + lane, g1 = g0 + 32;
+                if (g != lo) {
+                    if (g0 < hi) e0 = __ldg(m.gl + g0);
+                    if (g1 < hi) e1 = __ldg(m.gl + g1);
+                }
+                T x0, y0, z0, x1, y1, z1;
+                if (g0 < hi) {
+                    x0 = __ldcg(Lc + e0.x); y0 = __ldcg(Lc + e0.y);
+                    z0 = __ldcg((e0.z < ct ? v : Di) + e0.z);
+                }
+                if (g1 < hi) {
+                    x1 = __ldcg(Lc + e1.x); y1 = __ldcg(Lc + e1.y);
+                    z1 = __ldcg((e1.z < ct ? v : Di) + e1.z);
+                }
+                if (g0 < hi) s += x0 * (y0 * z0);
+                if (g1 < hi) s += x1 * (y1 * z1);
+            }
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) {
+                const T u = T(src) - s;
+                if (diag) {
+                    v[cc] = u;
+                    Di[cc] = pivot_recip(u);
+                    const double dd = double(u);
+                    if (!isfinite(dd)) atomicCAS(fstat, PF_OK, PF_ERR_NONFINITE);
+                    else if (fabs(dd) <= 1e-14 * amax) atomicCAS(fstat, PF_OK, PF_ERR_SINGULAR);
+                } else {
+                    Lc[p] = u;
+                }
+            }
+        }
+        ta = te;
+        te = tn;
+        if (ta + gw < te) fetch(ta + gw);
+        cluster_sync<C>();
+    }
+    for (int t = m.jlt[l0] + rank * int(blockDim.x) + int(threadIdx.x); t < tend; t += C * int(blockDim.x)) {
+        const int cc = m.jtcol[t - m.jg0];
+        if (cc < 0) continue;
+        const int p = t - cc - 1;
+        const T lv = __ldcg(Lc + p) * __ldcg(Di + cc);
+        Lc[p] = lv;
+        v[m.offLr + m.Cpos[p]] = lv;
+    }
+}
+
+// One cluster per instance, or (jobs) per matrix of a pack.
+constexpr int kTopThreads = 512;
+template <class T>
+__global__ void __launch_bounds__(kTopThreads)
+    k_factor_top(DevMat m, const double *A, T *F, int *fstatus, const double *amax, const FactorJob *jobs) {
+    const int inst = int(blockIdx.x) / kTailCtas, rank = int(cluster_rank());
+    if (jobs) {
+        const FactorJob &J = jobs[inst];
+        factor_top<T, kTailCtas>(J.m, J.A, static_cast<T *>(J.F), J.fstatus, *J.amax, rank);
+    } else {
+        factor_top<T, kTailCtas>(m, A + (long long)inst * m.stride, F + (long long)inst * m.stride, fstatus + inst,
+                                 amax[inst], rank);
+    }
+}
+
 // Tail values of the matrices of a pack (block-strided per job).
 template <class T>
 __global__ void k_tail_values_jobs(const FactorJob *jobs) {
@@ -1145,17 +1244,56 @@ cudaError_t launch_tail_values(const DevMat &m, int prec, const void *F, void *T
     return cudaGetLastError();
 }
 
+namespace {
+template <class T>
+cudaError_t launch_top(const DevMat &m, const double *A, T *F, int *fstatus, const double *amax,
+                       const FactorJob *jobs, int count, cudaStream_t s, int *resident = nullptr) {
+    cudaError_t e = cudaFuncSetAttribute(k_factor_top<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(unsigned(count) * kTailCtas);
+    cfg.blockDim = dim3(kTopThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kTailCtas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (resident) return cudaOccupancyMaxActiveClusters(resident, k_factor_top<T>, &cfg);
+    return cudaLaunchKernelEx(&cfg, k_factor_top<T>, m, A, F, fstatus, amax, jobs);
+}
+}  // namespace
+
+bool factor_top_fits(int prec) {
+    int n = 0;
+    const cudaError_t e =
+        prec == PF_FP64 ? launch_top<double>(DevMat(), nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, &n)
+                        : launch_top<float>(DevMat(), nullptr, nullptr, nullptr, nullptr, nullptr, 1, nullptr, &n);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && n > 0;
+}
+
 cudaError_t launch_factor_jobs(const FactorJob *jobs_dev, int njob, const int2 *items_dev,
-                               unsigned nitems, unsigned *sync_dev, int prec, int nsm, cudaStream_t s) {
+                               unsigned nitems, unsigned *sync_dev, int prec, int nsm, bool top, cudaStream_t s) {
     k_factor_prep_jobs<<<njob, 256, 0, s>>>(jobs_dev, sync_dev);
     long long blocks = (nitems + kDepThreads / 32 - 1) / (kDepThreads / 32);
     if (blocks > (long long)nsm * 2) blocks = (long long)nsm * 2;
     if (blocks < 1) blocks = 1;
     if (prec == PF_FP64) {
         k_factor_dep_jobs<double><<<int(blocks), kDepThreads, 0, s>>>(jobs_dev, items_dev, nitems, sync_dev, 0u);
+        if (top) {
+            const cudaError_t e = launch_top<double>(DevMat(), nullptr, nullptr, nullptr, nullptr, jobs_dev, njob, s);
+            if (e != cudaSuccess) return e;
+        }
         k_tail_values_jobs<double><<<dim3(8, unsigned(njob)), 256, 0, s>>>(jobs_dev);
     } else {
         k_factor_dep_jobs<float><<<int(blocks), kDepThreads, 0, s>>>(jobs_dev, items_dev, nitems, sync_dev, 0u);
+        if (top) {
+            const cudaError_t e = launch_top<float>(DevMat(), nullptr, nullptr, nullptr, nullptr, jobs_dev, njob, s);
+            if (e != cudaSuccess) return e;
+        }
         k_tail_values_jobs<float><<<dim3(8, unsigned(njob)), 256, 0, s>>>(jobs_dev);
     }
     return cudaGetLastError();
@@ -1243,7 +1381,8 @@ cudaError_t launch_factor(const DevMat &m, int prec, const double *A, void *F, i
         const size_t tsmem = factor_tail_smem(m, prec);
         const bool tail = fs.tail && m.ft_ng > 0 && m.ft_tmax >= 0 && fs.partg &&
                           tsmem + 1024 <= fs.smem_optin;
-        const int ncols = tail ? m.t0 : m.n;
+        const bool top = !tail && fs.top && m.jct[2] < m.n;
+        const int ncols = tail ? m.t0 : top ? m.jct[2] : m.n;
         const int per_sm = fs.blocks_per_sm > 0 && fs.blocks_per_sm < 2 ? fs.blocks_per_sm : 2;  // resident blocks per SM (registers)
         long long blocks = ((long long)ncols * ninst + kDepThreads / 32 - 1) / (kDepThreads / 32);
         if (blocks > (long long)fs.nsm * per_sm) blocks = (long long)fs.nsm * per_sm;
@@ -1259,6 +1398,7 @@ cudaError_t launch_factor(const DevMat &m, int prec, const double *A, void *F, i
                 e = launch_factor_tail<double>(m, static_cast<const double *>(fs.partg), static_cast<double *>(F),
                                                fstatus, fs.amax, ninst, tsmem, fs.tail_cluster, s);
             }
+            if (top) e = launch_top<double>(m, A, static_cast<double *>(F), fstatus, fs.amax, nullptr, ninst, s);
         } else {
             if (ncols > 0)
                 k_factor_dep<float><<<int(blocks), kDepThreads, 0, s>>>(m, A, static_cast<float *>(F),
@@ -1269,6 +1409,7 @@ cudaError_t launch_factor(const DevMat &m, int prec, const double *A, void *F, i
                 e = launch_factor_tail<float>(m, static_cast<const float *>(fs.partg), static_cast<float *>(F),
                                               fstatus, fs.amax, ninst, tsmem, fs.tail_cluster, s);
             }
+            if (top) e = launch_top<float>(m, A, static_cast<float *>(F), fstatus, fs.amax, nullptr, ninst, s);
         }
         return e != cudaSuccess ? e : cudaGetLastError();
     }

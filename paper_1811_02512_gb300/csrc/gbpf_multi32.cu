@@ -1,0 +1,15 @@
+// gbpf_multi32.cu -- the FP32 instantiations of gbpf_multi.cuh.
+#include "gbpf_multi.cuh"
+
+namespace gbpf {
+
+cudaError_t multi_run_f32(const MultiArgs &a, size_t smem, cudaStream_t s) {
+    return multi_run_t<float>(a, smem, s);
+}
+
+cudaError_t multi_pack_f32(const MultiArgs *args, const int *order, int ngrid, unsigned *counter, size_t smem,
+                           int blocks, cudaStream_t s) {
+    return multi_pack_t<float>(args, order, ngrid, counter, smem, blocks, s);
+}
+
+}  // namespace gbpf

@@ -1,0 +1,15 @@
+// gbpf_multi64.cu -- the FP64 instantiations of gbpf_multi.cuh.
+#include "gbpf_multi.cuh"
+
+namespace gbpf {
+
+cudaError_t multi_run_f64(const MultiArgs &a, size_t smem, cudaStream_t s) {
+    return multi_run_t<double>(a, smem, s);
+}
+
+cudaError_t multi_pack_f64(const MultiArgs *args, const int *order, int ngrid, unsigned *counter, size_t smem,
+                           int blocks, cudaStream_t s) {
+    return multi_pack_t<double>(args, order, ngrid, counter, smem, blocks, s);
+}
+
+}  // namespace gbpf

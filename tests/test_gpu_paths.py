@@ -54,6 +54,32 @@ def _flow(case, g, ncase, prec, tol=1e-11, **kw):
     return st, res, vm.cpu().numpy(), va.cpu().numpy()
 
 
+# Cases per block 1, 2 and 4 with a partial last block (152 SMs: 1
+# case each up to 152, 2 up to 304, then 4), load and outage cases, small
+# grids without and with a narrow top, and grids whose solve vector does not
+# fit shared memory (FP64 above about 27,000 rows).
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("n,ncase,nout", [(3, 1, 0), (37, 153, 0), (700, 307, 2), (1425, 613, 5), (30000, 2, 0)])
+def test_cases_per_block(oracle, n, ncase, nout, prec):
+    raw = gridgen.small_raw(n, 5) if n < 100 else gridgen.delaunay_raw(n, 5)
+    case = _loaded(raw, 1.0 / 256 if n > 5000 else 1.0 / 32)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    sc = gridgen.scenarios(case, n_load=ncase - nout, n_outage=nout, seed=3)
+    g = gbpf.Grid(case)
+    g.set_cases(ncase, sc.load_scale, sc.outage)
+    gbpf.pf_set_tuning(g.ctx, 1, 0, 0, 0, 2 if nout else 0, 0)
+    for ir_tol in (1e-3, 1e-10) if prec == "fp32" else (1e-10,):
+        st, res, vm, va = _flow(case, g, ncase, p, ir_tol=ir_tol)
+        assert st == gbpf.PF_OK and np.all(res["status"] == gbpf.PF_OK)
+        # every case's mismatch is within 1e-11; the state follows to the
+        # inverse Jacobian's norm times that, below 1e3 on these grids
+        for c in {0, 1 % ncase, ncase // 2, ncase - 1 - nout, ncase - 1}:
+            rc, vm0, va0, _, _ = oracle.power_flow(gridgen.apply_scenario(case, sc, c), oracle.NR, tol=1e-12)
+            assert rc == oracle.OK
+            assert np.abs(vm[c] - vm0).max() <= 1e-8 and np.abs(va[c] - va0).max() <= 1e-8
+    g.close()
+
+
 # Cases that leave the fixed-point range of the iteration (a slack angle
 # beyond it, a set-point beyond it) run on the FP64 form instead, beside
 # cases that stay; given starts are kept for them.
