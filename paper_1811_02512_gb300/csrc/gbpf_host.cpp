@@ -2173,6 +2173,10 @@ pf_status ensure_nr_storage(pf_ctx *ctx, int prec) {
         }
     }
     if (!w.jfstat[prec]) TRY(dalloc(ctx, &w.jfstat[prec], size_t(ctx->dc.ncase)));
+    {
+        MultiSteps steps;  // one case per block, no inverse of the top
+        TRY(ensure_multi_steps(ctx, PF_MAT_BP, prec, 1, false, steps));
+    }
     if (!w.jdone) {
         const size_t nd = size_t(ctx->dc.ncase) * size_t(std::max(1, m.n));
         TRY(dalloc(ctx, &w.jdone, nd));
@@ -2202,6 +2206,7 @@ NrLaunch nr_launch(pf_ctx *ctx, int prec) {
     L.cluster = nr_cluster_size(L.m, ctx->dc.ncase, ctx->num_sms, prec, ctx->smem_optin);
     L.jdone = w.jdone;
     L.jsync = w.jsync;
+    L.js = ctx->msteps[PF_MAT_BP][prec == PF_FP64 ? 1 : 0][0];
     return L;
 }
 

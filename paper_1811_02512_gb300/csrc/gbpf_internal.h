@@ -682,6 +682,7 @@ struct NrLaunch {
     unsigned *jdone = nullptr;  // [ncase][n] column done flags of the Jacobian factor
     unsigned *jsync = nullptr;  // [ncase][2] column counter, abort flag
     unsigned epoch0 = 0;        // factorisation k of this launch publishes epoch0 + k
+    MultiSteps js;              // steps of the substitutions (none: the staged sweeps)
 };
 cudaError_t launch_nr(const NrLaunch &L, cudaStream_t s);
 int nr_cluster_size(const DevMat &m, int ncase, int num_sms, int prec, size_t smem_optin);

@@ -306,6 +306,7 @@ void fill_nr_args(const NrLaunch &L, NrArgs &a) {
     a.gvm = L.gvm;
     a.dJdP = L.dJdP;
     a.dJdQ = L.dJdQ;
+    a.js = L.js;
     a.jdone = L.jdone;
     a.jsync = L.jsync;
     a.epoch0 = L.epoch0;
