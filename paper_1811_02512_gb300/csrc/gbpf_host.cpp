@@ -1703,7 +1703,7 @@ void free_case_storage(pf_ctx *ctx) {
         for (int b = 0; b < 2; b++) {
             dfree(ctx, w.fstatus[a][b]);
             w.fstatus[a][b] = nullptr;
-            w.factored[a][b] = false;
+            w.factored[a][b] = w.lazy[a][b] = false;
         }
     }
     for (int q = 0; q < 2; q++) {
@@ -1847,7 +1847,56 @@ pf_status factor_matrix(pf_ctx *ctx, int which, int prec, cudaStream_t s, int bl
         if (e != cudaSuccess) return cuda_fail(ctx, e, "tail inverse launch");
     }
     w.factored[which][prec] = true;
+    w.lazy[which][prec] = false;
     return PF_OK;
+}
+
+// The own factors that a run by rule left out (lazy), formed on `s`.
+pf_status own_factors(pf_ctx *ctx, int which, int prec, cudaStream_t s) {
+    if (ctx->ws.factored[which][prec] || !ctx->ws.lazy[which][prec]) return PF_OK;
+    return factor_matrix(ctx, which, prec, s);
+}
+
+// Whether every outaged branch of the batch leaves the grid connected (no
+// bridge of the in-service branches: Tarjan's low links).
+bool outages_connected(pf_ctx *ctx) {
+    const int n = ctx->nbus, m = ctx->nbr;
+    if (ctx->bridge.empty()) {
+        ctx->bridge.assign(std::max(1, m), 0);
+        std::vector<int> disc(n, -1), low(n, 0), pe(n, -1), at(n, 0), stack;
+        int timer = 0;
+        for (int root = 0; root < n; root++) {
+            if (disc[root] >= 0) continue;
+            disc[root] = low[root] = timer++;
+            at[root] = ctx->inc_ptr[root];
+            stack.assign(1, root);
+            while (!stack.empty()) {
+                const int v = stack.back();
+                if (at[v] < ctx->inc_ptr[v + 1]) {
+                    const int q = at[v]++, e = ctx->inc_br[q];
+                    if (e == pe[v] || !ctx->branch[e].status) continue;
+                    const int u = ctx->branch[e].from == v ? ctx->branch[e].to : ctx->branch[e].from;
+                    if (disc[u] < 0) {
+                        disc[u] = low[u] = timer++;
+                        pe[u] = e;
+                        at[u] = ctx->inc_ptr[u];
+                        stack.push_back(u);
+                    } else {
+                        low[v] = std::min(low[v], disc[u]);
+                    }
+                } else {
+                    stack.pop_back();
+                    if (!stack.empty()) {
+                        low[stack.back()] = std::min(low[stack.back()], low[v]);
+                        if (low[v] > disc[stack.back()]) ctx->bridge[pe[v]] = 1;
+                    }
+                }
+            }
+        }
+    }
+    for (int e : ctx->ws.case_out)
+        if (e >= 0 && ctx->bridge[e]) return false;
+    return true;
 }
 
 // Device tables of the several-cases-per-block kernel (see MultiNet).
@@ -2555,6 +2604,7 @@ pf_status pf_get_factor(pf_ctx *ctx, int32_t which, int32_t precision, int32_t c
     if (!ctx || (which != PF_MAT_BP && which != PF_MAT_BPP) ||
         (precision != PF_FP64 && precision != PF_FP32))
         return fail(ctx, PF_ERR_ARG, "bad matrix or precision");
+    TRY(own_factors(ctx, which, precision, nullptr));
     if (!ctx->ws.factored[which][precision]) return fail(ctx, PF_ERR_STATE, "not factored");
     if (c < 0 || c >= ctx->dc.ncase) return fail(ctx, PF_ERR_ARG, "case out of range");
     const DevMat &m = ctx->dm[which];
@@ -2592,6 +2642,7 @@ pf_status pf_solve(pf_ctx *ctx, int32_t which, int32_t precision, int32_t transp
     if (!ctx || (which != PF_MAT_BP && which != PF_MAT_BPP) || !rhs_inout_dev ||
         (precision != PF_FP64 && precision != PF_FP32))
         return fail(ctx, PF_ERR_ARG, "bad argument");
+    TRY(own_factors(ctx, which, precision, (cudaStream_t)stream));
     if (!ctx->ws.factored[which][precision]) return fail(ctx, PF_ERR_STATE, "pf_factor first");
     if (ncase < 1 || ncase > ctx->dc.ncase) return fail(ctx, PF_ERR_ARG, "ncase out of range");
     const void *F = precision == PF_FP64 ? (const void *)ctx->ws.F64[which]
@@ -2693,19 +2744,25 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     // k_fdpf's 16-block cluster shares only the nodal work (FP32, ir_tol 1e-3:
     // 0.27 ms against 0.55 on 200 buses, 0.87 against 1.35 on 2,643, 7.4
     // against 11.5 on 40,000; FP64 0.38 against 0.54, 11.1 against 14.6 on
-    // 40,000).
+    // 40,000).  Outage cases take the low-rank form for it when the tuning
+    // leaves the choice and no outage splits the grid (512 outages of a
+    // 1,425-bus grid: their own factors alone took 2.3 ms).
     MultiLaunch ml;
     const bool multi = (ctx->tune.tail == 0 || ctx->tune.tail == 3) &&
                        (ctx->tune.threads == 0 || ctx->tune.threads == 512) && ctx->tune.cluster <= 1;
-    if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2))
+    const bool by_rule = multi && ctx->tune.outage == 0 && ctx->dc.ninst > 1 && opts->flat_start &&
+                         !ctx->own_factors && outages_connected(ctx);
+    if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2 || by_rule))
         TRY(ensure_multi(ctx, prec, opts->ir_max > 0, ml));
-    const bool lowrank = ctx->tune.outage == 2 && ctx->dc.ninst > 1;
+    ctx->lowrank_by_rule = by_rule && ml.K > 0;
+    const bool lowrank = ctx->dc.ninst > 1 && (ctx->tune.outage == 2 || ctx->lowrank_by_rule);
     TRY(factor_both(ctx, prec, s, lowrank, false, ml.K > 0));
     if (lowrank) {
         TRY(prepare_lowrank(ctx, prec, s));
         // the outage instances' own factors were not computed: pf_solve and
         // pf_get_factor need pf_factor first
         w.factored[0][prec] = w.factored[1][prec] = false;
+        w.lazy[0][prec] = w.lazy[1][prec] = ctx->lowrank_by_rule;
     }
     const void *F0 = prec == PF_FP64 ? (const void *)w.F64[0] : (const void *)w.F32[0];
     const void *F1 = prec == PF_FP64 ? (const void *)w.F64[1] : (const void *)w.F32[1];
@@ -2772,6 +2829,7 @@ pf_status run_device_work(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, 
     if (graphs && ctx->gexec && key == ctx->gkey) {
         cudaError_t e = cudaGraphLaunch(ctx->gexec, s);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
+        ctx->lowrank_by_rule = ctx->graph_by_rule;
         for (int q = 0; q < PF_K_COUNT; q++) ctx->kstat[q].launches += ctx->glaunches[q];
         return PF_OK;
     }
@@ -2807,6 +2865,7 @@ pf_status run_device_work(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, 
         return issue_fdpf(ctx, opts, vm_dev, va_dev, engine, s);
     }
     ctx->gkey = key;
+    ctx->graph_by_rule = ctx->lowrank_by_rule;
     e = cudaGraphLaunch(ctx->gexec, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "graph launch");
     for (int q = 0; q < PF_K_COUNT; q++) ctx->kstat[q].launches += ctx->glaunches[q];
@@ -2905,6 +2964,18 @@ pf_status run_once(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, double 
                                     cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fdpf run");
+    if (engine == PF_ENGINE_BLOCK && ctx->lowrank_by_rule &&
+        std::any_of(res_host, res_host + ctx->dc.ncase, [](const pf_case_result &r) { return r.status != PF_OK; })) {
+        // a case that did not converge in the low-rank form by rule: the batch
+        // again with every outage's own factors, whose outcome stands
+        ctx->own_factors = true;
+        const pf_status st = issue_fdpf(ctx, opts, vm_dev, va_dev, engine, s);
+        ctx->own_factors = false;
+        if (st != PF_OK) return st;
+        e = cudaMemcpyAsync(res_host, w.res, sizeof(pf_case_result) * ctx->dc.ncase, cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "fdpf run");
+    }
     for (int c = 0; c < ctx->dc.ncase; c++)
         if (res_host[c].status != PF_OK)
             return fail(ctx, pf_status(res_host[c].status), "case %d: status %d after %d iterations (%s)",

@@ -421,6 +421,7 @@ struct Workspace {
     float *F32[2] = {nullptr, nullptr};
     int *fstatus[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}}; // [mat][prec] per instance
     bool factored[2][2] = {{false, false}, {false, false}};
+    bool lazy[2][2] = {{false, false}, {false, false}};  // own factors left out by a run: formed on demand
     int ninst_alloc = 0;
     // dependency-driven factor: per matrix, column-done flags [ninst][n]
     // (a column is done when its flag equals the epoch of the current
@@ -526,6 +527,10 @@ struct pf_ctx {
     int64_t glaunches[PF_K_COUNT] = {};
     bool graph_capturing = false;
     bool graphs_off = false;
+    // outage cases of a run by rule in their low-rank form (issue_fdpf): the
+    // last run took it, the captured graph does; own_factors: the run that
+    // repeats one with own factors
+    bool lowrank_by_rule = false, own_factors = false, graph_by_rule = false;
     int set_gen = 0;  // bumped by every pf_set_cases (the batch's arrays are new)
 };
 

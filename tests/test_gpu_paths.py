@@ -105,3 +105,47 @@ def test_leaves_the_fixed_point_range(oracle, shift, prec, engine):
     assert np.abs(vm[0].cpu().numpy() - vm0).max() <= 1e-7
     assert np.abs(va[0].cpu().numpy() - va0).max() <= 1e-7
     g.close()
+
+
+# Outage cases by rule in their low-rank form: with every outage's own factors
+# the same states, an outage that splits the grid reported as before, and the
+# own factors there for pf_solve and pf_get_factor afterwards.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_outages_by_rule(prec):
+    case = _loaded(gridgen.delaunay_raw(500, 21))
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    cut = gridgen.bridges(case.n, case.f, case.t, case.status)
+    ring = [k for k in range(case.m) if k not in set(cut)][:20]
+    out = np.array(ring + [-1, ring[0]], dtype=np.int32)
+
+    def run(branches, **tuning):
+        g = gbpf.Grid(case)
+        g.set_cases(len(branches), None, branches)
+        gbpf.pf_set_tuning(g.ctx, **tuning)
+        return (g,) + _flow(case, g, len(branches), p)
+
+    g, st, res, vm, va = run(out)
+    g1, st1, res1, vm1, va1 = run(out, outage=1)
+    assert st == st1 == gbpf.PF_OK and np.array_equal(res["iters"], res1["iters"])
+    # two runs of the same iteration: the difference is rounding, seen through
+    # the inverse matrices (FP32: their 1e-7, on steps that end at 1e-11)
+    assert np.abs(vm - vm1).max() <= 1e-10 and np.abs(va - va1).max() <= 1e-10
+    n = g.info.n[0]
+    rhs = torch.ones((len(out), n), dtype=torch.float64, device="cuda")
+    x, x1 = rhs.clone(), rhs.clone()
+    gbpf.pf_solve(g.ctx, gbpf.PF_MAT_BP, p, x, len(out))
+    gbpf.pf_solve(g1.ctx, gbpf.PF_MAT_BP, p, x1, len(out))
+    torch.cuda.synchronize()
+    assert torch.equal(x, x1)
+    assert all(np.array_equal(a, b) for a, b in zip(gbpf.pf_get_factor(g.ctx, 0, p, 3, g.info),
+                                                    gbpf.pf_get_factor(g1.ctx, 0, p, 3, g1.info)))
+    split = np.array([cut[0], -1], dtype=np.int32)
+    seen = []
+    for tuning in (dict(), dict(outage=1)):
+        g2, st2, res2, _, _ = run(split, **tuning)
+        assert st2 != gbpf.PF_OK and res2[0]["status"] == st2 and res2[1]["status"] == gbpf.PF_OK
+        if prec == "fp64":
+            assert st2 == gbpf.PF_ERR_SINGULAR
+        seen.append([tuple(r) for r in res2[["status", "iters", "method"]]])
+        g2.close()
+    assert seen[0] == seen[1]
