@@ -129,7 +129,8 @@ cudaError_t launch_pack(const PackGrid *grids, int ngrid, int prec, const pf_run
     // it fits; k_fdpf_pack below the others and what it left
     std::vector<MultiArgs> M(static_cast<size_t>(ngrid));
     size_t msmem = 0;
-    bool any = false;
+    bool any = false, wide = true;
+    int nbus_max = 0;
     for (int g = 0; g < ngrid; g++) {
         const PackGrid &p = grids[g];
         M[g].K = 0;
@@ -140,12 +141,16 @@ cudaError_t launch_pack(const PackGrid *grids, int ngrid, int prec, const pf_run
             } else {
                 msmem = need > msmem ? need : msmem;
                 any = true;
+                wide = wide && p.ml.C > 1;  // its solve vector has room for a cluster's
+                nbus_max = p.dn.nbus > nbus_max ? p.dn.nbus : nbus_max;
                 A[g].redo = p.ml.redo;
                 k_multi_rows<<<(p.dn.nbus + 127) / 128, 128, 0, s>>>(p.dn, p.ml.net, prec == PF_FP32 && o.ir_max > 0, o.tol);
             }
         }
         A[g].TW0 = A[g].TW1 = nullptr;
     }
+    const int C = any && wide ? multi_cluster_size(ngrid, nbus_max, nsm, prec, msmem) : 1;
+    for (MultiArgs &x : M) x.C = C;
     cudaError_t e = cudaMemcpyAsync(args_dev, A.data(), sizeof(RunArgs) * size_t(ngrid),
                                     cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)
@@ -159,8 +164,8 @@ cudaError_t launch_pack(const PackGrid *grids, int ngrid, int prec, const pf_run
         if (e != cudaSuccess) return e;
         const int blocks = ngrid < nsm ? ngrid : nsm;
         const MultiArgs *ma = static_cast<const MultiArgs *>(margs_dev);
-        e = prec == PF_FP64 ? multi_pack_f64(ma, order_dev, ngrid, counter_dev, msmem, blocks, s)
-                            : multi_pack_f32(ma, order_dev, ngrid, counter_dev, msmem, blocks, s);
+        e = prec == PF_FP64 ? multi_pack_f64(ma, order_dev, ngrid, counter_dev, msmem, blocks, C, s)
+                            : multi_pack_f32(ma, order_dev, ngrid, counter_dev, msmem, blocks, C, s);
         if (e != cudaSuccess) return e;
     }
     return launch_fdpf_pack(static_cast<const RunArgs *>(args_dev), order_dev, ngrid, counter_dev, prec,
@@ -175,6 +180,7 @@ size_t fill_multi_args(MultiArgs &ma, const RunArgs &a, const MultiLaunch &ml, c
     const int nmax = m[0].n > m[1].n ? m[0].n : m[1].n, nt = m[0].nt > m[1].nt ? m[0].nt : m[1].nt;
     ma.r = a;
     ma.K = ml.K;
+    ma.C = ml.C;
     ma.redo = ml.redo;
     ma.net = ml.net;
     ma.x = ml.x;
@@ -189,9 +195,35 @@ size_t fill_multi_args(MultiArgs &ma, const RunArgs &a, const MultiLaunch &ml, c
         ma.Kq[w] = w == 0 ? K0 : K1;
         ma.xs0[w] = m[w].n > nmax - ml.xs0 ? m[w].n - (nmax - ml.xs0) : 0;
     }
+    ma.xstride = ma.C > 1 ? nmax : ma.xs0[0] > ma.xs0[1] ? ma.xs0[0] : ma.xs0[1];
     ma.zoff = ((nmax - ml.xs0) * ma.K + 3) & ~3;  // 16-byte accesses
     ma.soff = int((elt * (size_t(ma.zoff) + size_t(nt) * size_t(ma.K)) + 15) & ~size_t(15));
-    return size_t(ma.soff) + sizeof(int2) * size_t(ma.steps[0].n() + ma.steps[1].n());
+    return multi_smem_bytes(ml, m, prec);
+}
+
+size_t multi_smem_bytes(const MultiLaunch &ml, const DevMat *m, int prec) {
+    const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
+    const int nmax = m[0].n > m[1].n ? m[0].n : m[1].n, nt = m[0].nt > m[1].nt ? m[0].nt : m[1].nt;
+    const size_t zoff = size_t((nmax - ml.xs0) * ml.K + 3) & ~size_t(3);
+    const size_t soff = (elt * (zoff + size_t(nt) * size_t(ml.K)) + 15) & ~size_t(15);
+    return soff + sizeof(int2) * size_t(ml.steps[0].n() + ml.steps[1].n());
+}
+
+// A case alone on a block leaves the chip idle: 16 or 8 blocks share its nodal
+// work while every case has its cluster at once.  The line: the cluster
+// barriers, about ten a half-iteration, cost what that saves at some 2,000
+// buses (one FP32 case, ir_tol 1e-10, cluster against block: 0.71 ms against
+// 0.57 on 1,000 buses, 0.88 against 0.85 on 2,000, 1.08 against 1.18 on 3,000,
+// 1.92 against 2.66 on 10,000, 7.1 against 10.9 on 40,000; FP64 8.6 against
+// 12.3 on 40,000; nine cases of 10,000 buses 2.05 against 2.66).
+int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem) {
+    constexpr int kMultiClBuses = 2500;
+    if (nbus < kMultiClBuses) return 1;
+    for (int C : {16, 8})
+        if (groups * C <= num_sms &&
+            (prec == PF_FP64 ? multi_clusters_f64(C, smem) : multi_clusters_f32(C, smem)) >= groups)
+            return C;
+    return 1;
 }
 
 size_t multi_args_bytes() { return sizeof(MultiArgs); }

@@ -2048,8 +2048,8 @@ pf_status ensure_multi_steps(pf_ctx *ctx, int which, int prec, int K, bool top, 
 }
 
 // The several-cases-per-block launch of this batch: its shape and storage (K
-// = 0: it does not apply).
-pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, MultiLaunch &ml) {
+// = 0: it does not apply); groups, nbus: see multi_cluster_size (0: no clusters).
+pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus, MultiLaunch &ml) {
     Workspace &w = ctx->ws;
     ml.K = multi_cases(ctx->dm, prec, ctx->dc.ncase, ctx->num_sms, ctx->smem_optin, &ml.xs0);
     if (ml.K == 0) return PF_OK;
@@ -2057,9 +2057,15 @@ pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, MultiLaunch &ml) {
     ml.net = ctx->mnet;
     for (int q = 0; q < 2; q++)
         TRY(ensure_multi_steps(ctx, q, prec, ml.K, ctx->dm[q].npf3 > 0, ml.steps[q]));
+    const size_t smem = multi_smem_bytes(ml, ctx->dm, prec);
+    if (smem + 1024 > ctx->smem_optin) {  // a grid of very many levels: its steps do not fit
+        ml.K = 0;
+        return PF_OK;
+    }
+    if (ml.K == 1 && groups > 0) ml.C = multi_cluster_size(groups, nbus, ctx->num_sms, prec, smem);
     if (!w.redo) TRY(dalloc(ctx, &w.redo, size_t(ctx->dc.ncase)));
     ml.redo = w.redo;
-    const size_t rows = size_t(ctx->dc.ncase) * size_t(ml.xs0);
+    const size_t rows = size_t(ctx->dc.ncase) * size_t(ml.C > 1 ? std::max(ctx->dm[0].n, ctx->dm[1].n) : ml.xs0);
     if (rows > w.mxg_count) {
         drop_graph(ctx);
         dfree(ctx, w.mxg);
@@ -2763,11 +2769,10 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     }
     // several cases per block, wherever all solves use the base factor and the
     // tuning names no other tail form, block size or cluster: faster than
-    // k_fdpf at every size tried, a single case on one SM included, where
-    // k_fdpf's 16-block cluster shares only the nodal work (FP32, ir_tol 1e-3:
-    // 0.27 ms against 0.55 on 200 buses, 0.87 against 1.35 on 2,643, 7.4
-    // against 11.5 on 40,000; FP64 0.38 against 0.54, 11.1 against 14.6 on
-    // 40,000).  Outage cases take the low-rank form for it when the tuning
+    // k_fdpf at every size tried, its 16-block cluster for one case included
+    // (FP32, ir_tol 1e-3: 0.27 ms against 0.55 on 200 buses, 0.87 against 1.35
+    // on 2,643, 4.8 against 11.5 on 40,000; FP64 0.38 against 0.54, 8.6
+    // against 14.6 on 40,000).  Outage cases take the low-rank form for it when the tuning
     // leaves the choice and no outage splits the grid (512 outages of a
     // 1,425-bus grid: their own factors alone took 2.3 ms).
     MultiLaunch ml;
@@ -2776,7 +2781,7 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     const bool by_rule = multi && ctx->tune.outage == 0 && ctx->dc.ninst > 1 && opts->flat_start &&
                          !ctx->own_factors && outages_connected(ctx);
     if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2 || by_rule))
-        TRY(ensure_multi(ctx, prec, opts->ir_max > 0, ml));
+        TRY(ensure_multi(ctx, prec, opts->ir_max > 0, ctx->tune.cluster == 0 ? ctx->dc.ncase : 0, ctx->nbus, ml));
     ctx->lowrank_by_rule = by_rule && ml.K > 0;
     const bool lowrank = ctx->dc.ninst > 1 && (ctx->tune.outage == 2 || ctx->lowrank_by_rule);
     TRY(factor_both(ctx, prec, s, lowrank, false, ml.K > 0));
@@ -3347,6 +3352,7 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<PackGrid> pg(static_cast<size_t>(ngrid));
     std::vector<FactorJob> jobs(static_cast<size_t>(2 * ngrid));
+    const int largest = pk->grids[size_t(pk->order[0])]->nbus;
     for (int g = 0; g < ngrid; g++) {
         pf_ctx *ctx = pk->grids[g];
         pf_status st = ensure_cases(ctx);
@@ -3370,7 +3376,7 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
         p.TW0 = w.TW[0][prec];
         p.TW1 = w.TW[1][prec];
         if (ctx->tune.tail == 0 || ctx->tune.tail == 3) {
-            st = ensure_multi(ctx, prec, opts->ir_max > 0, p.ml);
+            st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, p.ml);
             if (st != PF_OK) return pack_fail(pk, st, "grid %d: %s", g, ctx->err.c_str());
         }
         p.A0 = w.A[0];

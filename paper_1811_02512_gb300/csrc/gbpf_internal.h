@@ -405,10 +405,11 @@ struct MultiSteps {
 };
 struct MultiLaunch {
     int K = 0;
+    int C = 1;                 // blocks per case: a cluster, K = 1
     int xs0 = 0;               // rows of the solve vector kept in global memory
     int *redo = nullptr;       // [ncase]
     int2 *x = nullptr;         // [ncase][nbus]
-    void *xg = nullptr;        // [ncase][xs0] of the factor type
+    void *xg = nullptr;        // [ncase][xs0] of the factor type; with clusters [ncase][rows]
     MultiSteps steps[2];
     MultiNet net;
 };
@@ -620,6 +621,11 @@ struct NrLaunch;
 // Cases per block for a batch: as few as let every block run at once, as
 // many as fit shared memory at most; 0 where not even one does.
 int multi_cases(const DevMat *m, int prec, int ncase, int num_sms, size_t smem_optin, int *xs0);
+// Blocks per case for `groups` cases (or grids of a pack, the largest of nbus
+// buses) of one case per block each with `smem` bytes: 16, 8 or 1.
+int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem);
+// Dynamic shared memory of the launch.
+size_t multi_smem_bytes(const MultiLaunch &ml, const DevMat *m, int prec);
 // fb (optional): the Newton-Raphson launch that unconverged cases fall back
 // to inside the same launch (ignored when its factor scratch does not fit);
 // TW0/TW1 (optional): tail-inverse values of instance 0 (tail form 3).

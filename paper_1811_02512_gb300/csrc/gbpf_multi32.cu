@@ -3,13 +3,15 @@
 
 namespace gbpf {
 
+int multi_clusters_f32(int C, size_t smem) { return multi_clusters_t<float>(C, smem); }
+
 cudaError_t multi_run_f32(const MultiArgs &a, size_t smem, cudaStream_t s) {
     return multi_run_t<float>(a, smem, s);
 }
 
 cudaError_t multi_pack_f32(const MultiArgs *args, const int *order, int ngrid, unsigned *counter, size_t smem,
-                           int blocks, cudaStream_t s) {
-    return multi_pack_t<float>(args, order, ngrid, counter, smem, blocks, s);
+                           int groups, int C, cudaStream_t s) {
+    return multi_pack_t<float>(args, order, ngrid, counter, smem, groups, C, s);
 }
 
 }  // namespace gbpf

@@ -57,12 +57,14 @@ def _flow(case, g, ncase, prec, tol=1e-11, **kw):
 # Cases per block 1, 2 and 4 with a partial last block (152 SMs: 1
 # case each up to 152, 2 up to 304, then 4), load and outage cases, small
 # grids without and with a narrow top, and grids whose solve vector does not
-# fit shared memory (FP64 above about 27,000 rows).
+# fit shared memory (FP64 above about 27,000 rows).  From 2,500 buses a few
+# cases run on clusters: of 16 blocks up to 9 cases, of 8 up to 19.
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-@pytest.mark.parametrize("n,ncase,nout", [(3, 1, 0), (37, 153, 0), (700, 307, 2), (1425, 613, 5), (30000, 2, 0)])
+@pytest.mark.parametrize("n,ncase,nout", [(3, 1, 0), (37, 153, 0), (700, 307, 2), (1425, 613, 5), (30000, 2, 0),
+                                          (2500, 9, 2), (2503, 15, 2), (2800, 40, 2)])
 def test_cases_per_block(oracle, n, ncase, nout, prec):
     raw = gridgen.small_raw(n, 5) if n < 100 else gridgen.delaunay_raw(n, 5)
-    case = _loaded(raw, 1.0 / 256 if n > 5000 else 1.0 / 32)
+    case = _loaded(raw, 1.0 / 256 if n > 5000 else 1.0 / 64 if n > 1500 else 1.0 / 32)
     p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
     sc = gridgen.scenarios(case, n_load=ncase - nout, n_outage=nout, seed=3)
     g = gbpf.Grid(case)
@@ -149,3 +151,33 @@ def test_outages_by_rule(prec):
         seen.append([tuple(r) for r in res2[["status", "iters", "method"]]])
         g2.close()
     assert seen[0] == seen[1]
+
+
+# The grids of a pack on clusters (up to 19 grids, the largest of 2,500 buses
+# or more) and one to a block: the same states as each grid by itself.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("sizes", [(2500, 120, 2011), (40, 7, 300)])
+def test_pack_on_clusters(prec, sizes):
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    cases = [_loaded(gridgen.small_raw(n, 3) if n < 100 else gridgen.delaunay_raw(n, 3), 1.0 / 64) for n in sizes]
+    grids = [gbpf.Grid(c) for c in cases]
+    for g in grids:
+        g.set_cases(1)
+    pk = gbpf.Pack(grids)
+    opts = gbpf.run_opts(gbpf.PF_FDPF, p, tol=1e-11, ir_tol=1e-10, max_iter=300)
+    vm = torch.zeros(sum(sizes), dtype=torch.float64, device="cuda")
+    va = torch.zeros_like(vm)
+    st, res = pk.run(opts, vm, va)
+    assert st == gbpf.PF_OK and np.all(res["status"] == gbpf.PF_OK)
+    for c, n, off in zip(cases, sizes, pk.offset):
+        g = gbpf.Grid(c)
+        g.set_cases(1)
+        st, res, vm1, va1 = _flow(c, g, 1, p, ir_tol=1e-10, engine=gbpf.PF_ENGINE_BLOCK)
+        assert st == gbpf.PF_OK
+        # both mismatches are within 1e-11: the bound of test_cases_per_block
+        assert np.abs(vm[off:off + n].cpu().numpy() - vm1[0]).max() <= 1e-8
+        assert np.abs(va[off:off + n].cpu().numpy() - va1[0]).max() <= 1e-8
+        g.close()
+    pk.close()
+    for g in grids:
+        g.close()
