@@ -201,6 +201,19 @@ size_t fill_multi_args(MultiArgs &ma, const RunArgs &a, const MultiLaunch &ml, c
     return multi_smem_bytes(ml, m, prec);
 }
 
+cudaError_t launch_lowrank_z_multi(const MultiLaunch &ml, const DevNet &dn, const DevCases &dc, const DevMat *m, int which,
+                                   int prec, const void *F, const void *TV, const void *TW, void *Z, cudaStream_t s) {
+    RunArgs r = {};
+    r.dn = dn;
+    r.dc = dc;
+    (which == 0 ? r.F0 : r.F1) = F;
+    (which == 0 ? r.TV0 : r.TV1) = TV;
+    (which == 0 ? r.TW0 : r.TW1) = TW;
+    MultiArgs ma;
+    const size_t smem = fill_multi_args(ma, r, ml, m, nullptr, nullptr, nullptr, nullptr, prec);
+    return prec == PF_FP64 ? multi_lowrank_f64(ma, which, Z, smem, s) : multi_lowrank_f32(ma, which, Z, smem, s);
+}
+
 size_t multi_smem_bytes(const MultiLaunch &ml, const DevMat *m, int prec) {
     const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
     const int nmax = m[0].n > m[1].n ? m[0].n : m[1].n, nt = m[0].nt > m[1].nt ? m[0].nt : m[1].nt;

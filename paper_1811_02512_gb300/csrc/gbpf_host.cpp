@@ -2086,10 +2086,18 @@ pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus,
 
 // Low-rank outages: Z and K of every outage instance of both matrices from
 // the base factors (after factor_both with lowrank).
-pf_status prepare_lowrank(pf_ctx *ctx, int prec, cudaStream_t s) {
+pf_status prepare_lowrank(pf_ctx *ctx, int prec, bool multi, cudaStream_t s) {
     Workspace &w = ctx->ws;
     const int ninst = ctx->dc.ninst;
     const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
+    MultiLaunch zl;  // the solves for Z, several per block
+    if (multi) {
+        zl.K = multi_cases(ctx->dm, prec, 2 * (ninst - 1), ctx->num_sms, ctx->smem_optin, &zl.xs0);
+        if (zl.xs0 > 0) zl.K = 0;
+        for (int q = 0; q < 2 && zl.K > 0; q++)
+            TRY(ensure_multi_steps(ctx, q, prec, zl.K, ctx->dm[q].npf3 > 0, zl.steps[q]));
+        if (zl.K > 0 && multi_smem_bytes(zl, ctx->dm, prec) + 1024 > ctx->smem_optin) zl.K = 0;
+    }
     for (int m = 0; m < 2; m++) {
         const DevMat &D = ctx->dm[m];
         if (!w.LZ[m][prec]) {
@@ -2114,8 +2122,13 @@ pf_status prepare_lowrank(pf_ctx *ctx, int prec, cudaStream_t s) {
         const void *F = prec == PF_FP64 ? (const void *)w.F64[m] : (const void *)w.F32[m];
         const void *TV = ctx->tune.tail != 2 ? w.TV[m][prec] : nullptr;
         cudaError_t e = counted(ctx, PF_K_SOLVE, 2, s, [&] {
+            if (zl.K > 0) {
+                const cudaError_t z = launch_lowrank_z_multi(zl, ctx->dn, ctx->dc, ctx->dm, m, prec, F, TV, w.TW[m][prec],
+                                                             w.LZ[m][prec], s);
+                if (z != cudaSuccess) return z;
+            }
             return launch_lowrank(D, ctx->dn, ctx->dc, m, prec, F, TV, w.LZ[m][prec], w.LK[m],
-                                  w.Lscr[m][prec], w.fstatus[m][prec], ctx->smem_optin, s);
+                                  w.Lscr[m][prec], w.fstatus[m][prec], ctx->smem_optin, zl.K > 0, s);
         });
         if (e != cudaSuccess) return cuda_fail(ctx, e, "low-rank outages");
     }
@@ -2786,7 +2799,7 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     const bool lowrank = ctx->dc.ninst > 1 && (ctx->tune.outage == 2 || ctx->lowrank_by_rule);
     TRY(factor_both(ctx, prec, s, lowrank, false, ml.K > 0));
     if (lowrank) {
-        TRY(prepare_lowrank(ctx, prec, s));
+        TRY(prepare_lowrank(ctx, prec, ml.K > 0, s));
         // the outage instances' own factors were not computed: pf_solve and
         // pf_get_factor need pf_factor first
         w.factored[0][prec] = w.factored[1][prec] = false;

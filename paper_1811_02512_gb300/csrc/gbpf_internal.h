@@ -624,6 +624,10 @@ int multi_cases(const DevMat *m, int prec, int ncase, int num_sms, size_t smem_o
 // Blocks per case for `groups` cases (or grids of a pack, the largest of nbus
 // buses) of one case per block each with `smem` bytes: 16, 8 or 1.
 int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem);
+// The columns of Z of launch_lowrank, ml.K of them per block on instance 0's
+// factor with its top's inverse; z_done there.
+cudaError_t launch_lowrank_z_multi(const MultiLaunch &ml, const DevNet &dn, const DevCases &dc, const DevMat *m, int which,
+                                   int prec, const void *F, const void *TV, const void *TW, void *Z, cudaStream_t s);
 // Dynamic shared memory of the launch.
 size_t multi_smem_bytes(const MultiLaunch &ml, const DevMat *m, int prec);
 // fb (optional): the Newton-Raphson launch that unconverged cases fall back
@@ -645,7 +649,7 @@ cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, i
 // outage cases.  gvec: [2 (ninst - 1)][n] scratch of the factor type.
 cudaError_t launch_lowrank(const DevMat &m, const DevNet &dn, const DevCases &dc, int which, int prec,
                            const void *F, const void *TV, void *Z, double *Kd, void *gvec, int *status,
-                           size_t smem_optin, cudaStream_t s);
+                           size_t smem_optin, bool z_done, cudaStream_t s);
 int fdpf_cluster_size(int ncase, int num_sms, int prec, size_t smem_optin, int nmax);
 
 // One grid of a pack (uneven multi-grid batch): its device network, case,

@@ -1171,7 +1171,7 @@ cudaError_t launch_finite_check(const double *x, long long n, int *bad, cudaStre
 
 cudaError_t launch_lowrank(const DevMat &m, const DevNet &dn, const DevCases &dc, int which, int prec,
                            const void *F, const void *TV, void *Z, double *Kd, void *gvec, int *status,
-                           size_t smem_optin, cudaStream_t s) {
+                           size_t smem_optin, bool z_done, cudaStream_t s) {
     if (dc.ninst < 2) return cudaSuccess;
     const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
     const size_t ring = size_t(kStages) * kStageBytes;
@@ -1184,7 +1184,8 @@ cudaError_t launch_lowrank(const DevMat &m, const DevNet &dn, const DevCases &dc
     if (prec == PF_FP64) {
         e = cudaFuncSetAttribute(k_lowrank_z<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
-        k_lowrank_z<double><<<blocks, kSolveThreads, smem, s>>>(m, dn, dc, static_cast<const double *>(F),
+        if (!z_done)
+            k_lowrank_z<double><<<blocks, kSolveThreads, smem, s>>>(m, dn, dc, static_cast<const double *>(F),
                                                                 static_cast<const double *>(TV),
                                                                 static_cast<double *>(Z),
                                                                 static_cast<double *>(gvec), use_smem, status);
@@ -1192,7 +1193,8 @@ cudaError_t launch_lowrank(const DevMat &m, const DevNet &dn, const DevCases &dc
     } else {
         e = cudaFuncSetAttribute(k_lowrank_z<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
-        k_lowrank_z<float><<<blocks, kSolveThreads, smem, s>>>(m, dn, dc, static_cast<const float *>(F),
+        if (!z_done)
+            k_lowrank_z<float><<<blocks, kSolveThreads, smem, s>>>(m, dn, dc, static_cast<const float *>(F),
                                                                static_cast<const float *>(TV),
                                                                static_cast<float *>(Z),
                                                                static_cast<float *>(gvec), use_smem, status);

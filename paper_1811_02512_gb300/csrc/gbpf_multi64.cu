@@ -14,4 +14,8 @@ cudaError_t multi_pack_f64(const MultiArgs *args, const int *order, int ngrid, u
     return multi_pack_t<double>(args, order, ngrid, counter, smem, groups, C, s);
 }
 
+cudaError_t multi_lowrank_f64(const MultiArgs &a, int which, void *Z, size_t smem, cudaStream_t s) {
+    return multi_lowrank_t<double>(a, which, Z, smem, s);
+}
+
 }  // namespace gbpf

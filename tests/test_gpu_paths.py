@@ -112,12 +112,15 @@ def test_leaves_the_fixed_point_range(oracle, shift, prec, engine):
 # Outage cases by rule in their low-rank form: with every outage's own factors
 # the same states, an outage that splits the grid reported as before, and the
 # own factors there for pf_solve and pf_get_factor afterwards.
+# The low-rank data of 20, 90 and 157 outages is solved for 1, 2 and 4 columns
+# per block.
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-def test_outages_by_rule(prec):
-    case = _loaded(gridgen.delaunay_raw(500, 21))
+@pytest.mark.parametrize("count", [20, 90, 157])
+def test_outages_by_rule(prec, count):
+    case = _loaded(gridgen.delaunay_raw(500, 21), 1.0 / 64)
     p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
     cut = gridgen.bridges(case.n, case.f, case.t, case.status)
-    ring = [k for k in range(case.m) if k not in set(cut)][:20]
+    ring = [k for k in range(case.m) if k not in set(cut)][:count]
     out = np.array(ring + [-1, ring[0]], dtype=np.int32)
 
     def run(branches, **tuning):
