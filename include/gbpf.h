@@ -118,9 +118,10 @@ typedef struct {
                            storage on first use. */
 } pf_run_opts;
 
-/* Engines of pf_run_to_tol.  BLOCK: one thread block (or, for a few large
- * cases, a 16-block cluster) per case, each case iterating independently in
- * one persistent launch.  LANES (FDPF only): the batch advances in lockstep
+/* Engines of pf_run_to_tol.  BLOCK: 1, 2 or 4 cases per thread block (a few
+ * large cases: a cluster of 16 or 8 blocks per case), each case iterating
+ * independently in one persistent launch; one case per block where the
+ * solves use the case's own factors or the tuning says so.  LANES (FDPF only): the batch advances in lockstep
  * in groups of 32 cases, one case per lane; the mismatch, convergence test
  * and update run over (bus, case) pairs, each substitution over blocks of
  * 4, 2 or 1 cases whose vectors fit in shared memory, and one half-iteration
@@ -142,7 +143,7 @@ enum { PF_ENGINE_AUTO = 0, PF_ENGINE_BLOCK = 1, PF_ENGINE_LANES = 2, PF_ENGINE_C
  *   engine   PF_ENGINE_BLOCK, PF_ENGINE_LANES or PF_ENGINE_CLUSTER, used
  *            by FDPF runs whose options ask for PF_ENGINE_AUTO;
  *   cluster  thread blocks per case of a single-case FDPF run (1, 8, 16;
- *            capped at what fits the GPU); with engine PF_ENGINE_CLUSTER
+ *            capped at what fits the GPU; 0: by size); with engine PF_ENGINE_CLUSTER
  *            instead the subtree levels per step of its substitutions (1 to
  *            8, 0 = 3): g levels of a CTA's subtrees are solved in one step
  *            through the inverse of their block of L (formed after every
@@ -161,9 +162,11 @@ enum { PF_ENGINE_AUTO = 0, PF_ENGINE_BLOCK = 1, PF_ENGINE_LANES = 2, PF_ENGINE_C
  *            2: outage cases reuse the base factors with a low-rank
  *            (Woodbury) correction of each solve by the outaged branch's
  *            share (block engine; FP32 runs still refine against each
- *            case's exact matrix in FP64);
- *   threads  threads of each block of the block engine when it runs one
- *            block per case (512, 256 or 128): smaller blocks let more
+ *            case's exact matrix in FP64), 0: form 2 for a flat start when
+ *            no outage splits the grid (a batch in which a case fails is run
+ *            again in form 1), else 1;
+ *   threads  threads of each block of the block engine (512, 256 or 128; 256
+ *            and 128 always run one case per block): smaller blocks let more
  *            cases share an SM (2, 4 or 6 to 8), so that their latency-bound
  *            substitutions overlap one another's FP64 mismatch work; a
  *            block of 256 or 128 threads keeps its solve vector in global
