@@ -240,7 +240,7 @@ def measured_traffic(workload, prec_name, ncase, kernel):
     summary of the same kernel and workload (scaled by cases when the capture
     ran fewer cases), or None when there is no such capture."""
     files = {("plain10k", "fp64", "k_fdpf_cl"): "k_fdpf_cl_plain10k_fp64.md",
-             ("batch10k", "fp32", "k_fdpf"): "k_fdpf_batch128_fp32.md"}
+             ("batch10k", "fp32", "k_fdpf_multi"): "k_fdpf_multi_batch608_fp32.md"}
     name = files.get((workload, prec_name, kernel))
     if not name:
         return None
@@ -822,10 +822,15 @@ def main():
            "algorithmic_bytes_per_launch": alg_bytes}
     hbm["frac"] = hbm["achieved"] / hbm_peak
     engine_used = (tuning or {}).get("engine", engine)
-    kname = "k_fdpf_cl" if engine_used == gbpf.PF_ENGINE_CLUSTER else "k_fdpf"
+    tn = tuning or {}
+    # the several-cases-per-block kernel runs what the base factor can solve
+    multi = (tn.get("tail", 0) in (0, 3) and tn.get("threads", 0) in (0, 512) and tn.get("cluster", 0) <= 1
+             and (outage is None or tn.get("outage", 0) != 1))
+    kname = "k_fdpf_cl" if engine_used == gbpf.PF_ENGINE_CLUSTER else "k_fdpf_multi" if multi else "k_fdpf"
     hbm["traffic"] = measured_traffic(args.workload, prec_name, ncase, kname) if method == gbpf.PF_FDPF else None
     if ncase_all > 1:
-        # a batch is bound by the FP64 pipe (GB300 runs FP64 at 1/64 of FP32)
+        # a batch's arithmetic, whatever unit does it, against the FP64 pipe
+        # (GB300 runs FP64 at 1/64 of FP32; the nodal part runs in fixed point)
         solves64 = float(np.sum(res["iters"])) if prec == gbpf.PF_FP64 else 0.0
         flops = fp64_flops_per_launch(g.info, base, half_iters, resid, solves64)
         peak = fp64_peak_tflops(clk.get("sm_mhz"))
