@@ -45,7 +45,7 @@ __device__ __forceinline__ int4 fx_entry(double g, double b, int q) {
 // and the entry's fixed-point form.  Bound by latency: the indices of four
 // incident branches are read before their terms, three round trips to memory
 // (with the terms formed here, four FP64 divisions a branch in a row, a launch
-// took 18 to 22 us at any size up to 10,000 buses).
+// took 18 to 22 us at any size up to 10,000 buses; 8 us at 10,000 now).
 __device__ __forceinline__ void ybus_entry(const DevNet &dn, int t) {
     if (t < dn.nbus) {
         const int i = t, q1 = dn.inc_ptr[i + 1];
@@ -855,6 +855,7 @@ __global__ void __launch_bounds__(kFactorThreads)
 // units 2^-(q + 2).  A branch with an end outside the fixed-point range takes
 // the FP64 form.  Both ends' voltages are formed per branch rather than once
 // per bus: the call needs no scratch that calls on other streams share.
+// 13,500 branches x 256 cases: 168 us, 823 in FP64.
 __global__ void k_branch_flows(DevNet dn, DevCases dc, const double *vm, const double *va, int ncase,
                                double *flows) {
     const long long total = (long long)ncase * dn.nbr;
@@ -1098,7 +1099,8 @@ __device__ __forceinline__ double fx_mismatch(double spec, long long value, int 
     return fx_fits(spec, q) ? fx_to_double(fx_from_double(spec, q) - value, q) : spec - fx_to_double(value, q);
 }
 
-// 10,000 buses x 256 cases: 228 us in FP64.
+// 10,000 buses x 256 cases: 104 us and 42 for the voltages; 228 and 124 in
+// FP64.
 __global__ void k_mismatch_rows(DevNet dn, DevCases dc, const double *vm, const double *va, const int4 *ef,
                                 long long st, double *dp, double *dq, double *maxmis) {
     const int c = blockIdx.y;
