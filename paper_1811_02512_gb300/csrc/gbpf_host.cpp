@@ -3388,7 +3388,10 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
         p.TV1 = ctx->tune.tail != 2 ? w.TV[1][prec] : nullptr;
         p.TW0 = w.TW[0][prec];
         p.TW1 = w.TW[1][prec];
-        if (ctx->tune.tail == 0 || ctx->tune.tail == 3) {
+        // more grids than SMs: k_fdpf_pack keeps two grids on an SM, where
+        // this kernel's registers allow one (256 grids of 2,000 to 80,000 buses,
+        // FP32: 149 ms against 184; 100 grids 133 ms here, 137 there)
+        if (ngrid <= ctx->num_sms && (ctx->tune.tail == 0 || ctx->tune.tail == 3)) {
             st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, p.ml);
             if (st != PF_OK) return pack_fail(pk, st, "grid %d: %s", g, ctx->err.c_str());
         }
@@ -3447,7 +3450,8 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
     if (e == cudaSuccess)
         e = launch_factor_jobs(pk->jobs_dev, 2 * ngrid, pk->items_dev,
                                unsigned(top ? pk->n_below : pk->items.size()), pk->fsync, prec, pk->num_sms, top, s);
-    if (e == cudaSuccess)
+    const bool multi = std::any_of(pg.begin(), pg.end(), [](const PackGrid &p) { return p.ml.K > 0; });
+    if (e == cudaSuccess && multi)
         e = launch_tail_w_jobs(pk->jobs_dev, 2 * ngrid, pk->tw_first, pk->tw_blocks, pk->tw_depth, prec, s);
     if (e != cudaSuccess)
         return pack_fail(pk, e == cudaErrorMemoryAllocation ? PF_ERR_OOM : PF_ERR_CUDA, "pack factor: %s",

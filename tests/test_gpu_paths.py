@@ -157,9 +157,10 @@ def test_outages_by_rule(prec, count):
 
 
 # The grids of a pack on clusters (up to 19 grids, the largest of 2,500 buses
-# or more) and one to a block: the same states as each grid by itself.
+# or more), one to a block, and more grids than SMs: the same states as each
+# grid by itself.
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
-@pytest.mark.parametrize("sizes", [(2500, 120, 2011), (40, 7, 300)])
+@pytest.mark.parametrize("sizes", [(2500, 120, 2011), (40, 7, 300), (40, 7) * 77])
 def test_pack_on_clusters(prec, sizes):
     p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
     cases = [_loaded(gridgen.small_raw(n, 3) if n < 100 else gridgen.delaunay_raw(n, 3), 1.0 / 64) for n in sizes]
