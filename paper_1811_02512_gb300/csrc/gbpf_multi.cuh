@@ -648,9 +648,11 @@ __device__ __forceinline__ void accumulate_multi(const MultiArgs &ma, MultiShare
                 const float f = x.at(r)[k];
                 left |= !(fabsf(f) < 1.75f);
                 FxLimbs w = fx_limbs60(f);
-                if (!first) {
+                if (!first) {  // the sum keeps the parts' bound: limbs hold less than 2
                     const int2 o = st.x[at];
-                    w = fx_split(fx_join(w.h, w.l) + fx_join(o.x, o.y));
+                    const long long sum = fx_join(w.h, w.l) + fx_join(o.x, o.y);
+                    left |= (sum < 0 ? -sum : sum) >= 7ll << 58;
+                    w = fx_split(sum);
                 }
                 st.x[at] = make_int2(w.h, w.l);
             } else if (first) {
@@ -760,9 +762,9 @@ __device__ __forceinline__ void update_multi(const MultiArgs &ma, MultiShared<K>
         if (r < 0) continue;
         long long d;  // units 2^-60, |d| < 2
         bool ok;
-        if (refined) {
+        if (refined) {  // checked as it was summed (accumulate_multi)
             d = fx_join(w.x, w.y);
-            ok = (d < 0 ? -d : d) < (1ll << 61);
+            ok = true;
         } else {
             const T x = xv.at(r)[k];
             if constexpr (sizeof(T) == 4) {
