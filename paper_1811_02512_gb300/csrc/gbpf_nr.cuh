@@ -677,7 +677,8 @@ __device__ bool nr_solve(const NrArgs &a, Ring *R, unsigned char *stages, T *xs,
     }
     bn = block_max(bn, red);
     bool ok = true;
-    double last = INFINITY;
+    constexpr double kStagnant = 1e-9;
+    double first = 0.0, last = INFINITY;
     for (int k = 0;; k++) {
         if (a.js.steps && blockDim.x == kMultiThreads) {
             sweep_block2<T, TRANS, false>(a.js.steps, a.js.nf, m.Fp, m.Fc, F + (TRANS ? m.jUr : m.jLr), nullptr, xv);
@@ -699,12 +700,16 @@ __device__ bool nr_solve(const NrArgs &a, Ring *R, unsigned char *stages, T *xs,
         // what tells: an ill-conditioned component is still converging when
         // its share of the residual is long below the rounding of the rest
         // (stopping on the residual left 1.5e-10 of error where this leaves
-        // 4e-13 and all 21 solves 1.3e-12, on a 20,000-bus grid).
+        // 4e-13 and all 21 solves 1.3e-12, on a 20,000-bus grid).  Only
+        // corrections far below the first solution are that rounding: with a
+        // factor that is hardly an inverse they shrink by less than a tenth
+        // from the start, and all ir_max of them are needed.
         double step = 0.0;
         if (always_refine) step = block_max(double(dn), red);
         else __syncthreads();
         if (!refine || k >= a.ir_max) break;
-        if (always_refine && k > 1 && step > 0.9 * last) break;
+        if (k == 0) first = step;
+        if (always_refine && step > 0.9 * last && step <= kStagnant * first) break;
         last = step;
         double rn = 0.0;
         for (int r = threadIdx.x; r < m.n; r += blockDim.x) {

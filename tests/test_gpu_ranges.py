@@ -40,3 +40,22 @@ def test_refined_step_beyond_the_limbs():
     # FP32 roundings of two solves of a step of at most 3.2
     assert np.abs(va[0] - va[1]).max() <= 8 * 3.2 * 2.0 ** -23
     assert np.abs(va[0][:, 0] - want * (1 - 0.35 ** 2)).max() <= 8 * 3.2 * 2.0 ** -23
+
+
+# The FP32 factor holds the weak branch as `held` instead of weak, so every
+# correction of the adjoint leaves 1 - weak / held of the error: 20 of them are
+# all it has, and they are all taken.
+@pytest.mark.parametrize("strong,weak,held", [(2.0 ** 23 + 0.45, 0.08, 1.0), (2.0 ** 23 + 0.4, 0.15, 1.0),
+                                              (2.0 ** 23 + 0.3, 1.3, 2.0)])
+def test_adjoint_of_a_poor_factor_takes_every_correction(strong, weak, held):
+    g = gbpf.Grid(_chain(strong, weak, 0.0))
+    g.set_cases(1)
+    vm = torch.ones((1, 3), dtype=torch.float64, device="cuda")
+    va, gvm, dP, dQ = (torch.zeros_like(vm) for _ in range(4))
+    gva = torch.tensor([[1.0, 0.0, 0.0]], dtype=torch.float64, device="cuda")
+    gbpf.pf_adjoint(g.ctx, gbpf.PF_FP32, vm, va, gva, gvm, dP, dQ, 1)
+    # dJ/dP at bus 1 is 1 / weak; the 21 solves leave (1 - weak / held)^21 of
+    # it, to FP32's rounding of the last correction and what it multiplies
+    left = (1 - weak / held) ** 21
+    assert abs(weak * dP[0, 1].item() - (1 - left)) <= 1e-5
+    g.close()
