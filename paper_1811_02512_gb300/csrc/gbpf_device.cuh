@@ -873,12 +873,13 @@ constexpr int kFxNone = int(0x80000000u);
 // bus_current.  Twelve integer multiply-adds an entry, where the FP64 form
 // has four multiply-adds of 64 cycles: the nodal mismatch of the 10,000-bus
 // batch was bound by those.  CHECK: returns false when a voltage is kFxNone
-// (the outaged branch's other end is a neighbour too).
+// (the outaged branch's other end is a neighbour too) or the row is one for
+// FP64 (yst).
 template <bool CHECK>
 __device__ __forceinline__ bool fx_bus_current(const DevNet &dn, int i, int outage, const int4 *ef, int st,
                                                long long &ir_out, long long &ii_out) {
     FxAcc ir{0, 0}, ii{0, 0};
-    bool ok = !CHECK || dn.ysc[i] != kFxNoScale;
+    bool ok = !CHECK || dn.yst[i] != kFxNoScale;
     auto term = [&](const int4 &y, const int4 &v) {
         fx_mac(ir, y.x, y.y, v.x, v.y);
         fx_mac(ir, -y.z, -y.w, v.z, v.w);
@@ -1017,11 +1018,13 @@ __device__ __forceinline__ long long fx_mul60(long long a, long long b) {
 }
 
 // Bus states given by a caller may be out of the fixed-point range: their
-// entry is kFxNone, and what needs it takes the FP64 form.  An angle beyond
-// fx_sincos's range only goes through CUDA's sincos.
+// entry is kFxNone, and what needs it takes the FP64 form.  A small |V| is
+// out of it too: its e + jf would have fewer bits than a double (at 1e-6 a
+// flow was off by 1e-5 of itself).  An angle beyond fx_sincos's range only
+// goes through CUDA's sincos.
 __device__ __forceinline__ int4 fx_polar_any(double vm, double va) {
-    const unsigned h = unsigned(__double2hiint(vm)) & 0x7fffffffu, t = unsigned(__double2hiint(va)) & 0x7fffffffu;
-    if (h >= 0x3fff0000u || t >= 0x7ff00000u) return make_int4(kFxNone, 0, 0, 0);
+    const unsigned t = unsigned(__double2hiint(va)) & 0x7fffffffu;
+    if (!fx_vm_ok(vm) || t >= 0x7ff00000u) return make_int4(kFxNone, 0, 0, 0);
     if (t < 0x401f0000u) return fx_polar(vm, va);
     double s, c;
     sincos(va, &s, &c);

@@ -1577,8 +1577,8 @@ pf_status ensure_device(pf_ctx *ctx) {
         {
             // fixed-point rows and branch terms (see DevNet); fma() as the
             // device's own contraction, the same on every host
-            std::vector<double> bry(8 * size_t(std::max(1, nbranch)), 0.0), l1(nbus, 0.0);
-            std::vector<int> &ysc = ctx->ysc, yesc(dn.nnz);
+            std::vector<double> bry(8 * size_t(std::max(1, nbranch)), 0.0), l1(nbus, 0.0), lg(nbus, 0.0), lb(nbus, 0.0);
+            std::vector<int> &ysc = ctx->ysc, yesc(dn.nnz), yst(nbus);
             ysc.assign(nbus, 0);
             std::vector<int4> bryx(4 * size_t(std::max(1, nbranch)), int4{0, 0, 0, 0});
             auto fx_scale = [](double sum) {  // units 2^-q that take `sum` to at most 2^58
@@ -1597,8 +1597,12 @@ pf_status ensure_device(pf_ctx *ctx) {
                 o[3] = bc;
                 o[4] = -g / t;
                 o[5] = -b / t;
-                const int q = fx_scale(std::fabs(o[0]) + std::fabs(o[1]) + std::fabs(o[2]) + std::fabs(o[3]) +
-                                       std::fabs(o[4]) + std::fabs(o[5]));
+                double all = 0.0, least = INFINITY;
+                for (int k = 0; k < 6; k++) {
+                    all += std::fabs(o[k]);
+                    least = std::min(least, std::fabs(o[k]));
+                }
+                const int q = 48.0 * least >= all ? fx_scale(all) : kFxNoScale;
                 for (int k = 0; k < 3 && q != kFxNoScale; k++) {
                     const FxLimbs x = fx_split(fx_from_double(o[2 * k], q)), y = fx_split(fx_from_double(o[2 * k + 1], q));
                     bryx[4 * size_t(e) + k] = int4{x.h, x.l, y.h, y.l};
@@ -1613,14 +1617,22 @@ pf_status ensure_device(pf_ctx *ctx) {
                 l1[bf[e]] += std::fabs(o[0]) + std::fabs(g / (t * t)) + std::fabs(b / (t * t)) +
                              std::fabs(0.5 * bb[e] / (t * t)) + m;
                 l1[bt[e]] += std::fabs(o[2]) + std::fabs(g) + std::fabs(b) + std::fabs(0.5 * bb[e]) + m;
+                for (int s : {0, 1}) {
+                    lg[s ? bt[e] : bf[e]] += std::fabs(o[2 * s]) + std::fabs(o[4]);
+                    lb[s ? bt[e] : bf[e]] += std::fabs(o[2 * s + 1]) + std::fabs(o[5]);
+                }
             }
             for (int i = 0; i < nbus; i++) {
                 ysc[i] = fx_scale(l1[i] + std::fabs(gs[i]) + std::fabs(bs[i]));
+                const double g = lg[i] + std::fabs(gs[i]), b = lb[i] + std::fabs(bs[i]);
+                yst[i] = 16.0 * std::min(g, b) >= g + b ? ysc[i] : kFxNoScale;
+                dn.rows64 |= yst[i] == kFxNoScale;
                 for (int p = ctx->rowptr[i]; p < ctx->rowptr[i + 1]; p++) yesc[p] = ysc[i];
             }
             if ((st = upload(ctx, &dn.bry, bry.data(), bry.size()))) break;
             if ((st = upload(ctx, &dn.bryx, bryx.data(), bryx.size()))) break;
             if ((st = upload(ctx, &dn.ysc, ysc.data(), ysc.size()))) break;
+            if ((st = upload(ctx, &dn.yst, yst.data(), yst.size()))) break;
             if ((st = upload(ctx, &dn.yesc, yesc.data(), yesc.size()))) break;
             if ((st = dalloc(ctx, &dn.Yx, dn.nnz))) break;
         }

@@ -331,7 +331,18 @@ struct DevNet {
     // e's terms G_ff, B_ff, G_tt, B_tt, G_ft, B_ft (pi model), 1/x, 0, all zero
     // out of service; bryx[4 e
     // ..]: the same three pairs as limbs in units 2^-q, then {q, 0, 0, 0}.
-    int *ysc = nullptr, *yesc = nullptr;
+    // One unit for a row or branch holds its small terms with fewer bits than
+    // a double: the fixed-point sums are off by some 2^-59 of all magnitudes,
+    // an FP64 sum of P at a nearly flat state by 2^-53 of the conductances
+    // alone, of Q by 2^-53 of the susceptances.  The calls that evaluate given
+    // states take fixed point where neither share is below 1/16 of the row
+    // (yst[i] = ysc[i], else kFxNoScale; rows64: some row is), and none of a
+    // branch's six terms below 1/48 of their sum (q = kFxNoScale).  On a
+    // lossless branch between angles of 1e-6 the flow was off by 3e-13 of
+    // itself, behind a tap of 1e-3 by 2e-14, 2e-16 in FP64.  The iteration,
+    // which ends at a tolerance on the absolute mismatch, takes ysc.
+    int *ysc = nullptr, *yesc = nullptr, *yst = nullptr;
+    int rows64 = 0;
     int4 *Yx = nullptr, *bryx = nullptr;
     double *bry = nullptr;
 };
@@ -548,8 +559,10 @@ cudaError_t launch_assemble_slots(const DevNet &dn, const DevCases &dc, const De
 cudaError_t launch_branch_flows(const DevNet &dn, const DevCases &dc, const double *vm, const double *va,
                                 int ncase, double *flows, double *loss, cudaStream_t s);
 // e + jf of every case's state in fixed point (gbpf_fx.cuh) into the first
-// half of its ef region [4 nbus]; kFxNone where a voltage is out of range.
-cudaError_t launch_polar(const DevNet &dn, int ncase, const double *vm, const double *va, double *ef, cudaStream_t s);
+// half of its ef region [4 nbus]; kFxNone where a voltage is out of range;
+// with64: e and f in FP64 into the second half.
+cudaError_t launch_polar(const DevNet &dn, int ncase, const double *vm, const double *va, double *ef, bool with64,
+                         cudaStream_t s);
 struct FactorSync {
     unsigned *done = nullptr;  // [ninst][n]
     unsigned *sync = nullptr;  // [0] column counter, [1] abort flag

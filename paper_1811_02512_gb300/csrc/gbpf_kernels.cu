@@ -852,8 +852,8 @@ __global__ void __launch_bounds__(kFactorThreads)
 // the from side); zero for the case's outage and out-of-service branches.
 // From the end voltages in fixed point and the branch's terms (units 2^-q,
 // their sum at most 2^58): I_f and I_t in units 2^-(q + 1), the powers in
-// units 2^-(q + 2).  A branch with an end outside the fixed-point range takes
-// the FP64 form.  Both ends' voltages are formed per branch rather than once
+// units 2^-(q + 2).  A branch with an end outside the fixed-point range, or
+// with terms too far apart for one unit (see DevNet), takes the FP64 form.  Both ends' voltages are formed per branch rather than once
 // per bus: the call needs no scratch that calls on other streams share.
 // 13,500 branches x 256 cases: 168 us, 823 in FP64.
 __global__ void k_branch_flows(DevNet dn, DevCases dc, const double *vm, const double *va, int ncase,
@@ -1057,20 +1057,33 @@ __global__ void k_lowrank_k(DevMat m, DevNet dn, DevCases dc, int which, const T
 
 // ------------------------------------------------------------ Section II.A
 
-// e + jf of every bus of every case in fixed point, ef[c * st + i].
+// e + jf of every bus of every case in fixed point, ef[c * st + i]; with64: e
+// and f in FP64 behind them, [2][nbus].
+template <bool with64>
 __global__ void k_polar_to_rect(int nbus, int ncase, const double *vm, const double *va, int4 *ef, long long st) {
     const long long total = (long long)ncase * nbus;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
          idx += (long long)gridDim.x * blockDim.x) {
         const long long c = idx / nbus;
         ef[c * st + (idx - c * nbus)] = fx_polar_any(vm[idx], va[idx]);
+        if constexpr (with64) {
+            double *e = reinterpret_cast<double *>(ef + c * st + nbus) + (idx - c * nbus), sn, cs;
+            sincos(va[idx], &sn, &cs);
+            e[0] = vm[idx] * cs;
+            e[nbus] = vm[idx] * sn;
+        }
     }
 }
 
 // The FP64 form of (P, Q) at bus i of one case from its polar state, for rows
-// with a voltage outside the fixed-point range.
+// with a voltage outside the fixed-point range (grids with rows that always
+// take FP64 have e + jf in FP64 at hand, behind ef).
 __device__ __noinline__ void polar_injection(const DevNet &dn, int i, int outage, const double *vm, const double *va,
-                                             double &P, double &Q) {
+                                             const int4 *ef, double &P, double &Q) {
+    if (dn.rows64) {
+        const double *e = reinterpret_cast<const double *>(ef + dn.nbus);
+        return bus_injection(dn, i, outage, e, e + dn.nbus, P, Q);
+    }
     double s, c, ir = 0.0, ii = 0.0;
     for (int p = dn.rowptr[i]; p < dn.rowptr[i + 1]; p++) {
         const int k = dn.col[p];
@@ -1101,15 +1114,16 @@ __device__ __forceinline__ double fx_mismatch(double spec, long long value, int 
 
 // 10,000 buses x 256 cases: 104 us and 42 for the voltages; 228 and 124 in
 // FP64.
-__global__ void k_mismatch_rows(DevNet dn, DevCases dc, const double *vm, const double *va, const int4 *ef,
-                                long long st, double *dp, double *dq, double *maxmis) {
+__global__ void __launch_bounds__(256, 4)
+    k_mismatch_rows(DevNet dn, DevCases dc, const double *vm, const double *va, const int4 *ef, long long st, double *dp,
+                    double *dq, double *maxmis) {
     const int c = blockIdx.y;
     const int nbus = dn.nbus;
     const int4 *v = ef + c * st;
     const int outage = dc.outage[c];
     unsigned long long mx = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nbus; i += gridDim.x * blockDim.x) {
-        const int t = dn.btype[i], q = dn.ysc[i] + 2;
+        const int t = dn.btype[i], q = dn.yst[i] + 2;
         const long long idx = (long long)c * nbus + i;
         long long ir, ii;
         double a = 0.0, b = 0.0;
@@ -1118,7 +1132,7 @@ __global__ void k_mismatch_rows(DevNet dn, DevCases dc, const double *vm, const 
             if (t == PF_BUS_PQ) b = fx_mismatch(dc.Qsp[idx], fx_power(true, v[i], ir, ii), q);
         } else {
             double P, Q;
-            polar_injection(dn, i, outage, vm + (long long)c * nbus, va + (long long)c * nbus, P, Q);
+            polar_injection(dn, i, outage, vm + (long long)c * nbus, va + (long long)c * nbus, v, P, Q);
             if (t != PF_BUS_SLACK) a = dc.Psp[idx] - P;
             if (t == PF_BUS_PQ) b = dc.Qsp[idx] - Q;
         }
@@ -1485,10 +1499,13 @@ cudaError_t launch_selftest_sweep(const DevMat &m, int prec, const void *F, cons
     return cudaGetLastError();
 }
 
-// e + jf of every case's state into the first half of its ef region.
-cudaError_t launch_polar(const DevNet &dn, int ncase, const double *vm, const double *va, double *ef, cudaStream_t s) {
-    k_polar_to_rect<<<grid_for((long long)ncase * dn.nbus, 256), 256, 0, s>>>(
-        dn.nbus, ncase, vm, va, reinterpret_cast<int4 *>(ef), 2LL * dn.nbus);
+// e + jf of every case's state into the first half of its ef region; with64:
+// in FP64 into the second.
+cudaError_t launch_polar(const DevNet &dn, int ncase, const double *vm, const double *va, double *ef, bool with64,
+                         cudaStream_t s) {
+    auto *k = with64 ? k_polar_to_rect<true> : k_polar_to_rect<false>;
+    k<<<grid_for((long long)ncase * dn.nbus, 256), 256, 0, s>>>(dn.nbus, ncase, vm, va, reinterpret_cast<int4 *>(ef),
+                                                                2LL * dn.nbus);
     return cudaGetLastError();
 }
 
@@ -1497,7 +1514,7 @@ cudaError_t launch_mismatch(const DevNet &dn, const DevCases &dc, const double *
                             cudaStream_t s) {
     cudaError_t e = cudaMemsetAsync(maxmis, 0, sizeof(double) * ncase, s);
     if (e != cudaSuccess) return e;
-    e = launch_polar(dn, ncase, vm, va, ef, s);
+    e = launch_polar(dn, ncase, vm, va, ef, dn.rows64 != 0, s);
     if (e != cudaSuccess) return e;
     dim3 grid((dn.nbus + 255) / 256, ncase);
     k_mismatch_rows<<<grid, 256, 0, s>>>(dn, dc, vm, va, reinterpret_cast<const int4 *>(ef), 2LL * dn.nbus, dp, dq,

@@ -361,7 +361,7 @@ cudaError_t launch_nr(const NrLaunch &L, cudaStream_t s) {
 
 cudaError_t launch_objective(const DevNet &dn, const DevCases &dc, const double *vm, const double *va,
                              double *ef, double *J, double *gva, double *gvm, cudaStream_t s) {
-    cudaError_t e = launch_polar(dn, dc.ncase, vm, va, ef, s);
+    cudaError_t e = launch_polar(dn, dc.ncase, vm, va, ef, false, s);
     if (e != cudaSuccess) return e;
     const int nblk = (dn.nbus + 255) / 256;  // parts of J per case, after the case's e + jf
     k_objective<<<unsigned(nblk) * unsigned(dc.ncase), 256, 0, s>>>(dn, dc, vm, va, ef, gva, gvm);
