@@ -1577,7 +1577,8 @@ pf_status ensure_device(pf_ctx *ctx) {
         {
             // fixed-point rows and branch terms (see DevNet); fma() as the
             // device's own contraction, the same on every host
-            std::vector<double> bry(8 * size_t(std::max(1, nbranch)), 0.0), l1(nbus, 0.0), lg(nbus, 0.0), lb(nbus, 0.0);
+            std::vector<double> bry(8 * size_t(std::max(1, nbranch)), 0.0), l1(nbus, 0.0), lg(nbus, 0.0), lb(nbus, 0.0),
+                bp(nbus, 0.0);
             std::vector<int> &ysc = ctx->ysc, yesc(dn.nnz), yst(nbus);
             ysc.assign(nbus, 0);
             std::vector<int4> bryx(4 * size_t(std::max(1, nbranch)), int4{0, 0, 0, 0});
@@ -1620,6 +1621,7 @@ pf_status ensure_device(pf_ctx *ctx) {
                 for (int s : {0, 1}) {
                     lg[s ? bt[e] : bf[e]] += std::fabs(o[2 * s]) + std::fabs(o[4]);
                     lb[s ? bt[e] : bf[e]] += std::fabs(o[2 * s + 1]) + std::fabs(o[5]);
+                    bp[s ? bt[e] : bf[e]] += 2.0 * std::fabs(o[6]);
                 }
             }
             for (int i = 0; i < nbus; i++) {
@@ -1627,6 +1629,7 @@ pf_status ensure_device(pf_ctx *ctx) {
                 const double g = lg[i] + std::fabs(gs[i]), b = lb[i] + std::fabs(bs[i]);
                 yst[i] = 16.0 * std::min(g, b) >= g + b ? ysc[i] : kFxNoScale;
                 dn.rows64 |= yst[i] == kFxNoScale;
+                ctx->row_max = std::max(ctx->row_max, std::max(g + b, bp[i]));
                 for (int p = ctx->rowptr[i]; p < ctx->rowptr[i + 1]; p++) yesc[p] = ysc[i];
             }
             if ((st = upload(ctx, &dn.bry, bry.data(), bry.size()))) break;
@@ -2057,6 +2060,18 @@ pf_status ensure_multi_steps(pf_ctx *ctx, int which, int prec, int K, bool top, 
     }
     out = S;
     return PF_OK;
+}
+
+// Whether that kernel can refine as far as a run asks.  Its residual and its
+// solution are held to absolute units, some 2^-59 of a row's absolute sum: a
+// target below that is never seen to be met, and every solve then took all
+// ir_max corrections (ir_tol 1e-10, ir_abs 1e-30 on 700 buses: 55 corrections
+// against 16 with k_fdpf's FP64 residual).  The smallest target: ir_abs, or
+// ir_tol of a right-hand side at the tolerance.
+bool multi_refines(const pf_ctx *ctx, const pf_run_opts *o) {
+    if (o->precision != PF_FP32 || o->ir_max == 0) return true;
+    const double least = std::max(o->ir_abs > 0 ? o->ir_abs : 0.01 * o->tol, o->ir_tol * o->tol);
+    return least >= std::ldexp(ctx->row_max, -58);
 }
 
 // The several-cases-per-block launch of this batch: its shape and storage (K
@@ -2802,7 +2817,8 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     // 1,425-bus grid: their own factors alone took 2.3 ms).
     MultiLaunch ml;
     const bool multi = (ctx->tune.tail == 0 || ctx->tune.tail == 3) &&
-                       (ctx->tune.threads == 0 || ctx->tune.threads == 512) && ctx->tune.cluster <= 1;
+                       (ctx->tune.threads == 0 || ctx->tune.threads == 512) && ctx->tune.cluster <= 1 &&
+                       multi_refines(ctx, opts);
     const bool by_rule = multi && ctx->tune.outage == 0 && ctx->dc.ninst > 1 && opts->flat_start &&
                          !ctx->own_factors && outages_connected(ctx);
     if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2 || by_rule))
@@ -3403,7 +3419,7 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
         // more grids than SMs: k_fdpf_pack keeps two grids on an SM, where
         // this kernel's registers allow one (256 grids of 2,000 to 80,000 buses,
         // FP32: 149 ms against 184; 100 grids 133 ms here, 137 there)
-        if (ngrid <= ctx->num_sms && (ctx->tune.tail == 0 || ctx->tune.tail == 3)) {
+        if (ngrid <= ctx->num_sms && (ctx->tune.tail == 0 || ctx->tune.tail == 3) && multi_refines(ctx, opts)) {
             st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, p.ml);
             if (st != PF_OK) return pack_fail(pk, st, "grid %d: %s", g, ctx->err.c_str());
         }

@@ -513,6 +513,7 @@ struct pf_ctx {
     std::vector<int> ydiag, inc_ptr, inc_br, inc_side, inc_pos, br_pos, yoff_br;
     std::vector<int4> yoff;
     std::vector<int> mis_ord, mis_ord_cl, ysc;
+    double row_max = 0.0;      // largest absolute sum of a row of the admittance matrix, B' or B''
     std::vector<char> bridge;  // per branch: its outage splits the grid (on first use)
     int device = 0;
     int num_sms = 0;

@@ -167,3 +167,30 @@ def test_states_outside_the_range(special):
             gv[c] += 2 * gk * (vm[c] - vm[a] / tk * np.cos(dth))
         for got, want in ((gva, gt), (gvm, gv)):
             assert np.all(np.abs(got - want) <= 64 * 2.0 ** -53 * (row + 1.0))
+
+
+# Refinement asked for below the unit of the fixed-point residual (absolute
+# targets of 1e-30 on rows that sum to 174): as many corrections as the form
+# with the FP64 residual takes, alone and in a pack.
+@pytest.mark.parametrize("ir_tol,ir_abs", [(1e-10, 0.0), (1e-10, 1e-30), (1e-14, 1e-30), (1e-3, 1e-30)])
+def test_refinement_below_the_unit(ir_tol, ir_abs):
+    case = gridgen.delaunay_raw(700, 5).scaled_network(1.0 / 32)
+    opts = gbpf.run_opts(gbpf.PF_FDPF, gbpf.PF_FP32, tol=1e-8, ir_max=20, ir_tol=ir_tol, ir_abs=ir_abs)
+    steps = []
+    for tuning in (dict(cluster=1, tail=1, threads=512), dict(), None):
+        g = gbpf.Grid(case)
+        g.set_cases(1)
+        vm = torch.zeros((1, case.n), dtype=torch.float64, device="cuda")
+        va = torch.zeros_like(vm)
+        if tuning is None:
+            pk = gbpf.Pack([g])
+            st, res = pk.run(opts, vm[0], va[0])
+            pk.close()
+        else:
+            gbpf.pf_set_tuning(g.ctx, engine=gbpf.PF_ENGINE_BLOCK, **tuning)
+            st, res = gbpf.pf_run_to_tol(g.ctx, opts, vm, va, 1)
+        assert st == gbpf.PF_OK
+        steps.append(int(res["ir_steps"][0]))
+        g.close()
+    # a solve whose residual lies at the target may go either way: one in ten
+    assert max(steps) <= 1.1 * steps[0] + 2, steps
