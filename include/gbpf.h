@@ -163,8 +163,8 @@ enum { PF_ENGINE_AUTO = 0, PF_ENGINE_BLOCK = 1, PF_ENGINE_LANES = 2, PF_ENGINE_C
  *            (Woodbury) correction of each solve by the outaged branch's
  *            share (block engine; FP32 runs still refine against each
  *            case's exact matrix in FP64), 0: form 2 for a flat start when
- *            no outage splits the grid (a batch in which a case fails is run
- *            again in form 1), else 1;
+ *            no outage splits the grid (outage cases that do not converge are
+ *            run again in form 1, whose outcome stands), else 1;
  *   threads  threads of each block of the block engine (512, 256 or 128; 256
  *            and 128 always run one case per block): smaller blocks let more
  *            cases share an SM (2, 4 or 6 to 8), so that their latency-bound

@@ -95,7 +95,8 @@ void fill_run_args(RunArgs &a, const DevNet &dn, const DevCases &dc, const DevMa
     a.res = res;
     a.use_smem = 0;
     a.fallback = 0;
-    a.redo = nullptr;
+    a.redo = a.list = a.own_now = nullptr;
+    a.nlist = 0;
 }
 
 size_t run_args_bytes() { return sizeof(RunArgs); }
@@ -263,9 +264,12 @@ cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, i
                         double *xg, double *bmax, pf_case_result *res, size_t smem_optin,
                         size_t smem_per_sm, int cluster, int threads, cudaStream_t s, const void *Z0,
                         const void *Z1, const double *K0, const double *K1, const NrLaunch *fb,
-                        const void *TW0, const void *TW1, const int *redo, const MultiLaunch *multi) {
+                        const void *TW0, const void *TW1, const MultiLaunch *multi, const int *list, int nlist) {
     RunArgs a;
-    a.redo = redo;
+    a.redo = nullptr;
+    a.list = list;
+    a.nlist = nlist;
+    a.own_now = multi && multi->K > 0 ? multi->own_now : nullptr;
     a.Z0 = Z0;
     a.Z1 = Z1;
     a.K0 = K0;

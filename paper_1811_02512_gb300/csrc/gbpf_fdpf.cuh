@@ -51,6 +51,13 @@ struct RunArgs {
     // after k_fdpf_multi (or null): per case 0 done, 1 to be run, 2 its
     // fallback only
     const int *redo;
+    // the cases of the launch, nlist of them (null: all)
+    const int *list;
+    int nlist;
+    // low-rank outages by rule (or null): outage cases do not end here but
+    // with their own factors later -- those marked at once, the others if they
+    // leave the fixed-point range or take more than kOwnLaterHalf steps
+    const int *own_now;
 };
 
 
@@ -397,14 +404,15 @@ __global__ void __launch_bounds__(kRunThreads, C == 1 ? 2 : 1) k_fdpf(const __gr
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ double red[33];
     __shared__ Ring R;
-    const int c = int(blockIdx.x) / C, redo = a.redo ? a.redo[c] : 1;  // the same in a case's cluster
+    const int b = int(blockIdx.x) / C, c = a.list ? a.list[b] : b;
+    const int redo = a.redo ? a.redo[c] : 1;  // the same in a case's cluster
     if (redo == 0) return;
     if (redo == 2) {
         ring_init(&R);
         nr_fallback<T, C>(a.nr, c, C == 1 ? 0 : int(cluster_rank()), smem_raw, red, &R);
         return;
     }
-    fdpf_case<T, C>(a, int(blockIdx.x) / C, smem_raw, red, R, true);
+    fdpf_case<T, C>(a, c, smem_raw, red, R, true);
 }
 
 // Uneven multi-grid batch: one persistent launch over the grids of a pack,
@@ -455,7 +463,7 @@ cudaError_t launch_fdpf_t(const RunArgs &a, size_t smem, int threads, cudaStream
                                          int(smem));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(unsigned(a.dc.ncase) * C);
+    cfg.gridDim = dim3(unsigned(a.list ? a.nlist : a.dc.ncase) * C);
     cfg.blockDim = dim3(unsigned(threads));
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;

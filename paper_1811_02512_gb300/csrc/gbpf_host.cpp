@@ -1742,6 +1742,10 @@ void free_case_storage(pf_ctx *ctx) {
     dfree(ctx, w.iv); w.iv = nullptr;
     dfree(ctx, w.cstatus); w.cstatus = nullptr;
     dfree(ctx, w.redo); w.redo = nullptr;
+    dfree(ctx, w.own_now); w.own_now = nullptr;
+    dfree(ctx, w.own_set); w.own_set = nullptr;
+    w.own_case.clear();
+    w.own_key.clear();
     dfree(ctx, w.mx); w.mx = nullptr;
     dfree(ctx, w.mxg); w.mxg = nullptr; w.mxg_count = 0;
     dfree(ctx, w.res); w.res = nullptr;
@@ -1781,9 +1785,9 @@ pf_status assemble_matrix(pf_ctx *ctx, int which, int prec, cudaStream_t s, int 
 pf_status factor_job(pf_ctx *ctx, int which, int prec, FactorJob &J, cudaStream_t s) {
     Workspace &w = ctx->ws;
     const DevMat &m = ctx->dm[which];
+    const size_t flags = size_t(w.ninst_full) * size_t(std::max(1, m.n)) * sizeof(unsigned);
     if (++w.fepoch[which] >= kGraphEpoch) {
-        cudaError_t z = cudaMemsetAsync(w.fdone[which], 0,
-                                        size_t(ctx->dc.ninst) * size_t(std::max(1, m.n)) * sizeof(unsigned), s);
+        cudaError_t z = cudaMemsetAsync(w.fdone[which], 0, flags, s);
         if (z != cudaSuccess) return cuda_fail(ctx, z, "factor flags");
         w.fepoch[which] = 1u;
     }
@@ -1818,15 +1822,14 @@ pf_status factor_matrix(pf_ctx *ctx, int which, int prec, cudaStream_t s, int bl
     fs.done = w.fdone[which];
     fs.sync = w.fsync[which];
     fs.amax = w.famax[which];
+    const size_t flags = size_t(w.ninst_full) * size_t(std::max(1, m.n)) * sizeof(unsigned);
     if (ctx->graph_capturing) {  // every replay clears the flags and publishes kGraphEpoch
-        cudaError_t z = cudaMemsetAsync(w.fdone[which], 0,
-                                        size_t(ctx->dc.ninst) * size_t(std::max(1, m.n)) * sizeof(unsigned), s);
+        cudaError_t z = cudaMemsetAsync(w.fdone[which], 0, flags, s);
         if (z != cudaSuccess) return cuda_fail(ctx, z, "factor flags");
         fs.epoch = kGraphEpoch;
     } else {
         if (++w.fepoch[which] >= kGraphEpoch) {  // wrapped: clear the flags, restart at 1
-            cudaError_t z = cudaMemsetAsync(w.fdone[which], 0,
-                                            size_t(ctx->dc.ninst) * size_t(std::max(1, m.n)) * sizeof(unsigned), s);
+            cudaError_t z = cudaMemsetAsync(w.fdone[which], 0, flags, s);
             if (z != cudaSuccess) return cuda_fail(ctx, z, "factor flags");
             w.fepoch[which] = 1u;
         }
@@ -2605,6 +2608,7 @@ pf_status pf_set_cases(pf_ctx *ctx, int32_t ncase, const double *load_scale,
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e != cudaSuccess) return cuda_fail(ctx, e, "case spec");
         if (bad) return fail(ctx, PF_ERR_ARG, "non-finite load scale");
+        w0.own_key.clear();
         return PF_OK;
     }
     if (load_scale)
@@ -2616,7 +2620,7 @@ pf_status pf_set_cases(pf_ctx *ctx, int32_t ncase, const double *load_scale,
     free_case_storage(ctx);
     DevCases &dc = ctx->dc;
     dc.ncase = ncase;
-    dc.ninst = int(inst_out.size());
+    dc.ninst = w0.ninst_full = int(inst_out.size());
     TRY(upload(ctx, &dc.outage, out.data(), out.size()));
     TRY(upload(ctx, &dc.inst, inst.data(), inst.size()));
     TRY(upload(ctx, &dc.inst_outage, inst_out.data(), inst_out.size()));
@@ -2655,6 +2659,7 @@ pf_status pf_set_injections(pf_ctx *ctx, const double *psp_dev, const double *qs
     cudaError_t e = cudaMemcpyAsync(ctx->dc.Psp, psp_dev, bytes, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->dc.Qsp, qsp_dev, bytes, cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "set injections");
+    ctx->ws.own_key.clear();
     return PF_OK;
 }
 
@@ -2760,6 +2765,30 @@ pf_status pf_run_to_tol(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, do
 }  // extern "C"
 
 namespace {
+// The Newton-Raphson launch that a fast decoupled run's unconverged cases
+// switch to from a flat start inside the iteration launch (Section III).
+pf_status fallback_launch(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, double *va_dev, cudaStream_t s,
+                          NrLaunch &fbl) {
+    Workspace &w = ctx->ws;
+    TRY(ensure_nr_storage(ctx, opts->precision));
+    fbl = nr_launch(ctx, opts->precision);
+    fbl.o = *opts;
+    fbl.o.method = PF_NR;
+    fbl.o.max_iter = kFallbackIters;
+    fbl.o.flat_start = 1;
+    fbl.vm = vm_dev;
+    fbl.va = va_dev;
+    if (ctx->graph_capturing) {  // every replay clears the flags and counts from kNrGraphEpoch
+        cudaError_t e = cudaMemsetAsync(
+            w.jdone, 0, size_t(ctx->dc.ncase) * size_t(std::max(1, ctx->dm[0].n)) * sizeof(unsigned), s);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "fallback flags");
+        fbl.epoch0 = kNrGraphEpoch;
+    } else {
+        fbl.epoch0 = nr_epochs(ctx, unsigned(kFallbackIters) + 2u, s);
+    }
+    return PF_OK;
+}
+
 // Device work of one fast decoupled run on the block or the cluster engine,
 // enqueued on s without any host synchronisation: the admittance matrix,
 // B' and B'' assembled and factorised (B'' on the side stream), then the
@@ -2769,27 +2798,10 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     Workspace &w = ctx->ws;
     const int prec = opts->precision;
     TRY(assemble_ybus(ctx, s));
-    // FDPF -> NR fallback (Section III): unconverged cases switch to
-    // Newton-Raphson from a flat start inside the iteration launch
     NrLaunch fbl;
     const NrLaunch *fb = nullptr;
     if (opts->fallback) {
-        TRY(ensure_nr_storage(ctx, prec));
-        fbl = nr_launch(ctx, prec);
-        fbl.o = *opts;
-        fbl.o.method = PF_NR;
-        fbl.o.max_iter = kFallbackIters;
-        fbl.o.flat_start = 1;
-        fbl.vm = vm_dev;
-        fbl.va = va_dev;
-        if (ctx->graph_capturing) {  // every replay clears the flags and counts from kNrGraphEpoch
-            cudaError_t e = cudaMemsetAsync(
-                w.jdone, 0, size_t(ctx->dc.ncase) * size_t(std::max(1, ctx->dm[0].n)) * sizeof(unsigned), s);
-            if (e != cudaSuccess) return cuda_fail(ctx, e, "fallback flags");
-            fbl.epoch0 = kNrGraphEpoch;
-        } else {
-            fbl.epoch0 = nr_epochs(ctx, unsigned(kFallbackIters) + 2u, s);
-        }
+        TRY(fallback_launch(ctx, opts, vm_dev, va_dev, s, fbl));
         fb = &fbl;
     }
     if (engine == PF_ENGINE_CLUSTER) {
@@ -2820,16 +2832,24 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
                        (ctx->tune.threads == 0 || ctx->tune.threads == 512) && ctx->tune.cluster <= 1 &&
                        multi_refines(ctx, opts);
     const bool by_rule = multi && ctx->tune.outage == 0 && ctx->dc.ninst > 1 && opts->flat_start &&
-                         !ctx->own_factors && outages_connected(ctx);
+                         outages_connected(ctx);
     if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2 || by_rule))
         TRY(ensure_multi(ctx, prec, opts->ir_max > 0, ctx->tune.cluster == 0 ? ctx->dc.ncase : 0, ctx->nbus, ml));
     ctx->lowrank_by_rule = by_rule && ml.K > 0;
+    if (ctx->lowrank_by_rule) {
+        if (!w.own_now) {
+            TRY(dalloc(ctx, &w.own_now, size_t(ctx->dc.ncase)));
+            const cudaError_t e = cudaMemsetAsync(w.own_now, 0, sizeof(int) * size_t(ctx->dc.ncase), s);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "outage marks");
+        }
+        ml.own_now = w.own_now;
+    }
     const bool lowrank = ctx->dc.ninst > 1 && (ctx->tune.outage == 2 || ctx->lowrank_by_rule);
     TRY(factor_both(ctx, prec, s, lowrank, false, ml.K > 0));
     if (lowrank) {
         TRY(prepare_lowrank(ctx, prec, ml.K > 0, s));
         // the outage instances' own factors were not computed: pf_solve and
-        // pf_get_factor need pf_factor first
+        // pf_get_factor need pf_factor first, or form them on demand (by rule)
         w.factored[0][prec] = w.factored[1][prec] = false;
         w.lazy[0][prec] = w.lazy[1][prec] = ctx->lowrank_by_rule;
     }
@@ -2849,12 +2869,80 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
                            lowrank ? w.LZ[0][prec] : nullptr,
                            lowrank ? w.LZ[1][prec] : nullptr, lowrank ? w.LK[0] : nullptr,
                            lowrank ? w.LK[1] : nullptr, fb, tw ? w.TW[0][prec] : nullptr,
-                           tw ? w.TW[1][prec] : nullptr, nullptr, &ml);
+                           tw ? w.TW[1][prec] : nullptr, &ml);
     });
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fdpf launch");
     return PF_OK;
 }
 
+
+// The outage cases that a run by rule left, with their own factors, after that
+// run's results are in res_host: the base and the instances of these cases
+// alone are factorised (into the first slots) and k_fdpf runs the cases, with
+// the fallback where the run has it.  Their outcome is that of a run with own
+// factors throughout.  Runs of the same arguments and loads send them here at
+// once (own_now).  512 outages of 1,425 buses in FP64, one of which does not
+// converge: 11.3 ms (12.6 the first time), 21.2 when the whole batch ran again,
+// 14.3 with own factors from the start; with all of them failing 31.9, 56.7 and
+// 31.4 ms; one failing load case, which runs once, 10.3 and 24.2 ms.
+pf_status run_outages_again(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, double *va_dev,
+                            pf_case_result *res_host, cudaStream_t s) {
+    Workspace &w = ctx->ws;
+    const int ncase = ctx->dc.ncase, prec = opts->precision;
+    w.own_case.resize(size_t(ncase), 0);
+    std::vector<int> list, inst(size_t(ncase), 0), outs(1, -1);
+    bool more = false;
+    for (int c = 0; c < ncase; c++) {
+        if (w.case_out[c] < 0 || res_host[c].status == PF_OK) continue;
+        more |= !w.own_case[c];
+        w.own_case[c] = 1;
+        list.push_back(c);
+        inst[c] = int(outs.size());
+        outs.push_back(w.case_out[c]);
+    }
+    if (list.empty()) return PF_OK;
+    const int n = int(list.size());
+    if (!w.own_set) TRY(dalloc(ctx, &w.own_set, size_t(2 * ncase + w.ninst_full)));
+    auto put = [&](int *dst, const std::vector<int> &v) {
+        return cudaMemcpyAsync(dst, v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice, s);
+    };
+    int *inst_dev = w.own_set + ncase, *outs_dev = inst_dev + ncase;
+    cudaError_t e = put(w.own_set, list);
+    if (e == cudaSuccess) e = put(inst_dev, inst);
+    if (e == cudaSuccess) e = put(outs_dev, outs);
+    if (e == cudaSuccess && more) e = put(w.own_now, w.own_case);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "outage cases");
+    const DevCases all = ctx->dc;
+    ctx->dc.inst = inst_dev;
+    ctx->dc.inst_outage = outs_dev;
+    ctx->dc.ninst = n + 1;
+    NrLaunch fbl;
+    pf_status st = opts->fallback ? fallback_launch(ctx, opts, vm_dev, va_dev, s, fbl) : PF_OK;
+    if (st == PF_OK) st = factor_both(ctx, prec, s, false);
+    if (st == PF_OK) {
+        const void *F[2] = {prec == PF_FP64 ? (const void *)w.F64[0] : (const void *)w.F32[0],
+                            prec == PF_FP64 ? (const void *)w.F64[1] : (const void *)w.F32[1]};
+        const int cl = ctx->tune.cluster == 1 ? 1
+                                              : fdpf_cluster_size(n, ctx->num_sms, prec, ctx->smem_optin,
+                                                                  std::max(ctx->dm[0].n, ctx->dm[1].n));
+        e = counted(ctx, PF_K_RUN, 1, s, [&] {
+            return launch_fdpf(ctx->dn, ctx->dc, ctx->dm, prec, F[0], F[1], w.TV[0][prec], w.TV[1][prec], w.A[0],
+                               w.A[1], w.fstatus[0][prec], w.fstatus[1][prec], *opts, vm_dev, va_dev, w.ef, w.iv,
+                               w.vec, w.bmax, w.res, ctx->smem_optin, ctx->smem_per_sm, cl, 0, s, nullptr, nullptr,
+                               nullptr, nullptr, opts->fallback ? &fbl : nullptr, nullptr, nullptr, nullptr,
+                               w.own_set, n);
+        });
+        if (e != cudaSuccess) st = cuda_fail(ctx, e, "fdpf launch");
+    }
+    ctx->dc = all;
+    // the slots hold other instances than the batch's
+    w.factored[0][prec] = w.factored[1][prec] = false;
+    w.lazy[0][prec] = w.lazy[1][prec] = true;
+    if (st != PF_OK) return st;
+    e = cudaMemcpyAsync(res_host, w.res, sizeof(pf_case_result) * size_t(ncase), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? PF_OK : cuda_fail(ctx, e, "fdpf run");
+}
 
 // The device work of a run, from a CUDA graph when the same arguments come
 // again: the first call with a set of arguments runs directly (allocating
@@ -2894,6 +2982,14 @@ pf_status run_device_work(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, 
     put(t, sizeof(t));
     const int extra[3] = {engine, ctx->set_gen, ctx->dc.ncase};
     put(extra, sizeof(extra));
+    if (key != ctx->ws.own_key) {  // other arguments or loads: no case is known to need its own factors
+        ctx->ws.own_key = key;
+        if (std::count(ctx->ws.own_case.begin(), ctx->ws.own_case.end(), 1) > 0) {
+            ctx->ws.own_case.assign(ctx->ws.own_case.size(), 0);
+            const cudaError_t e = cudaMemsetAsync(ctx->ws.own_now, 0, sizeof(int) * ctx->ws.own_case.size(), s);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "outage marks");
+        }
+    }
     const bool graphs = !ctx->profiling && !ctx->graphs_off;
     if (graphs && ctx->gexec && key == ctx->gkey) {
         cudaError_t e = cudaGraphLaunch(ctx->gexec, s);
@@ -3033,18 +3129,8 @@ pf_status run_once(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, double 
                                     cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "fdpf run");
-    if (engine == PF_ENGINE_BLOCK && ctx->lowrank_by_rule &&
-        std::any_of(res_host, res_host + ctx->dc.ncase, [](const pf_case_result &r) { return r.status != PF_OK; })) {
-        // a case that did not converge in the low-rank form by rule: the batch
-        // again with every outage's own factors, whose outcome stands
-        ctx->own_factors = true;
-        const pf_status st = issue_fdpf(ctx, opts, vm_dev, va_dev, engine, s);
-        ctx->own_factors = false;
-        if (st != PF_OK) return st;
-        e = cudaMemcpyAsync(res_host, w.res, sizeof(pf_case_result) * ctx->dc.ncase, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "fdpf run");
-    }
+    if (engine == PF_ENGINE_BLOCK && ctx->lowrank_by_rule)
+        TRY(run_outages_again(ctx, opts, vm_dev, va_dev, res_host, s));
     for (int c = 0; c < ctx->dc.ncase; c++)
         if (res_host[c].status != PF_OK)
             return fail(ctx, pf_status(res_host[c].status), "case %d: status %d after %d iterations (%s)",

@@ -419,6 +419,7 @@ struct MultiLaunch {
     int C = 1;                 // blocks per case: a cluster, K = 1
     int xs0 = 0;               // rows of the solve vector kept in global memory
     int *redo = nullptr;       // [ncase]
+    const int *own_now = nullptr;  // [ncase] marks of RunArgs::own_now
     int2 *x = nullptr;         // [ncase][nbus]
     void *xg = nullptr;        // [ncase][xs0] of the factor type; with clusters [ncase][rows]
     MultiSteps steps[2];
@@ -434,7 +435,6 @@ struct Workspace {
     int *fstatus[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}}; // [mat][prec] per instance
     bool factored[2][2] = {{false, false}, {false, false}};
     bool lazy[2][2] = {{false, false}, {false, false}};  // own factors left out by a run: formed on demand
-    int ninst_alloc = 0;
     // dependency-driven factor: per matrix, column-done flags [ninst][n]
     // (a column is done when its flag equals the epoch of the current
     // factorisation), the column counter and abort flag, diagonal maxima
@@ -461,6 +461,13 @@ struct Workspace {
     double *iv = nullptr;     // [ncase][nbus] 1 / V
     int *cstatus = nullptr;   // [ncase] run status
     int *redo = nullptr;      // [ncase] marks of k_fdpf_multi
+    // outage cases by rule (issue_fdpf): those that go to their own factors at
+    // once, as of the last run of the same arguments; the second launch's case
+    // list, instances and their outages
+    int *own_now = nullptr, *own_set = nullptr;
+    std::vector<int> own_case;
+    std::vector<unsigned char> own_key;  // those arguments (run_device_work), empty: loads changed
+    int ninst_full = 0;       // instances that the factor storage is for
     int2 *mx = nullptr;       // [ncase][nbus] its refined solutions (FP32)
     void *mxg = nullptr;      // [ncase][rows in global memory] of 8 bytes
     size_t mxg_count = 0;
@@ -541,9 +548,8 @@ struct pf_ctx {
     bool graph_capturing = false;
     bool graphs_off = false;
     // outage cases of a run by rule in their low-rank form (issue_fdpf): the
-    // last run took it, the captured graph does; own_factors: the run that
-    // repeats one with own factors
-    bool lowrank_by_rule = false, own_factors = false, graph_by_rule = false;
+    // last run took it, the captured graph does
+    bool lowrank_by_rule = false, graph_by_rule = false;
     int set_gen = 0;  // bumped by every pf_set_cases (the batch's arrays are new)
 };
 
@@ -646,7 +652,8 @@ cudaError_t launch_lowrank_z_multi(const MultiLaunch &ml, const DevNet &dn, cons
 size_t multi_smem_bytes(const MultiLaunch &ml, const DevMat *m, int prec);
 // fb (optional): the Newton-Raphson launch that unconverged cases fall back
 // to inside the same launch (ignored when its factor scratch does not fit);
-// TW0/TW1 (optional): tail-inverse values of instance 0 (tail form 3).
+// TW0/TW1 (optional): tail-inverse values of instance 0 (tail form 3); list
+// (optional): the cases to run, on the device.
 cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, int prec,
                         const void *F0, const void *F1, const void *TV0, const void *TV1,
                         const double *A0, const double *A1,
@@ -656,8 +663,8 @@ cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, i
                         int threads, cudaStream_t s,
                         const void *Z0 = nullptr, const void *Z1 = nullptr, const double *K0 = nullptr,
                         const double *K1 = nullptr, const NrLaunch *fb = nullptr,
-                        const void *TW0 = nullptr, const void *TW1 = nullptr, const int *redo = nullptr,
-                        const MultiLaunch *multi = nullptr);
+                        const void *TW0 = nullptr, const void *TW1 = nullptr, const MultiLaunch *multi = nullptr,
+                        const int *list = nullptr, int nlist = 0);
 // Z = A^-1 U and K = (I - S U^T Z)^-1 S of every outage instance of matrix
 // `which` from the base factor F (instance 0): the low-rank form of the
 // outage cases.  gvec: [2 (ninst - 1)][n] scratch of the factor type.

@@ -1,0 +1,77 @@
+"""GPU checks of the mappings that a run takes by rule: the same outcome as the
+mapping set by hand."""
+import numpy as np
+import pytest
+
+from paper_1811_02512_gb300 import gbpf, gridgen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def _run(g, n, ncase, prec, **kw):
+    vm = torch.zeros((ncase, n), dtype=torch.float64, device="cuda")
+    va = torch.zeros_like(vm)
+    st, res = gbpf.pf_run_to_tol(g.ctx, gbpf.run_opts(gbpf.PF_FDPF, prec, **kw), vm, va, ncase)
+    return st, res, vm.cpu().numpy(), va.cpu().numpy()
+
+
+def _launches(g, kind):
+    return gbpf.pf_get_profile(g.ctx, kind, reset=True)[0]
+
+
+# Outage batches with cases that do not converge: those alone run again, with
+# their own factors, in the first call and in later ones (captured too); a load
+# case that fails does not make them.  The outcome is that of own factors for
+# every outage; what converged in the low-rank form is the same to rounding.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("fallback", [0, 1])
+@pytest.mark.parametrize("bad", [(), (3,), (0, 40, 119), (5, 121), (121,), tuple(range(120))])
+def test_outages_that_fail(bad, fallback, prec):
+    case = gridgen.delaunay_raw(300, 21).scaled_network(1.0 / 64)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    cut = set(gridgen.bridges(case.n, case.f, case.t, case.status))
+    out = np.array([k for k in range(case.m) if k not in cut][:120] + [-1, -1], np.int32)
+    ncase = len(out)
+    ls = np.ones((ncase, case.n))
+    for b in bad:
+        ls[b] *= 3000.0
+    own = gbpf.Grid(case)
+    own.set_cases(ncase, ls, out)
+    gbpf.pf_set_tuning(own.ctx, outage=1)
+    kw = dict(tol=1e-10, max_iter=60, fallback=fallback)
+    st1, res1, vm1, va1 = _run(own, case.n, ncase, p, **kw)
+    g = gbpf.Grid(case)
+    g.set_cases(ncase, ls, out)
+    fine = np.array([c not in bad for c in range(ncase)])
+    again = any(out[b] >= 0 for b in bad)
+    seen = []
+    for call in range(4):
+        _launches(g, gbpf.PF_K_RUN)
+        st, res, vm, va = _run(g, case.n, ncase, p, **kw)
+        assert _launches(g, gbpf.PF_K_RUN) == 1 + again, call
+        assert (st == gbpf.PF_OK) == (len(bad) == 0) == (st1 == gbpf.PF_OK)
+        assert np.array_equal(res["status"], res1["status"]) and np.array_equal(res["method"], res1["method"])
+        assert np.abs(res["iters"] - res1["iters"])[fine].max(initial=0) <= 1
+        # two mismatches of at most 1e-10, seen through the inverse Jacobian (below 1e3 here)
+        assert np.abs(vm[fine] - vm1[fine]).max(initial=0) <= 1e-7 and np.abs(va[fine] - va1[fine]).max(initial=0) <= 1e-7
+        seen.append((res, vm, va))
+    for res, vm, va in seen[1:]:
+        assert all(np.array_equal(res[f], seen[0][0][f]) for f in ("status", "iters", "ir_steps", "method"))
+        assert np.array_equal(vm, seen[0][1], equal_nan=True) and np.array_equal(va, seen[0][2], equal_nan=True)
+    # the batch's own factors for pf_solve, whatever the slots held
+    n = g.info.n[1]
+    x, x1 = (torch.ones((ncase, n), dtype=torch.float64, device="cuda") for _ in range(2))
+    gbpf.pf_solve(g.ctx, gbpf.PF_MAT_BPP, p, x, ncase)
+    gbpf.pf_solve(own.ctx, gbpf.PF_MAT_BPP, p, x1, ncase)
+    torch.cuda.synchronize()
+    assert torch.equal(x, x1)
+    # ordinary loads for the same outages: every case in the low-rank form again
+    g.set_cases(ncase, np.ones((ncase, case.n)), out)
+    for _ in range(2):
+        _launches(g, gbpf.PF_K_RUN)
+        st, res, vm, va = _run(g, case.n, ncase, p, **kw)
+        assert st == gbpf.PF_OK and np.all(res["method"] == gbpf.PF_FDPF)
+    assert _launches(g, gbpf.PF_K_RUN) == 1
+    g.close()
+    own.close()
