@@ -1746,6 +1746,7 @@ void free_case_storage(pf_ctx *ctx) {
     dfree(ctx, w.own_set); w.own_set = nullptr;
     w.own_case.clear();
     w.own_key.clear();
+    w.no_room = false;
     dfree(ctx, w.mx); w.mx = nullptr;
     dfree(ctx, w.mxg); w.mxg = nullptr; w.mxg_count = 0;
     dfree(ctx, w.res); w.res = nullptr;
@@ -2114,12 +2115,42 @@ pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus,
     return PF_OK;
 }
 
+// Storage of the low-rank form of the batch's outages.
+pf_status ensure_lowrank(pf_ctx *ctx, int prec) {
+    Workspace &w = ctx->ws;
+    const size_t ninst = size_t(ctx->dc.ninst);
+    for (int m = 0; m < 2; m++) {
+        const size_t n = size_t(std::max(1, ctx->dm[m].n));
+        auto make = [&](auto *t) -> pf_status {
+            if (!w.LZ[m][prec]) TRY(dalloc(ctx, &t, ninst * 2 * n));
+            if (!w.LZ[m][prec]) w.LZ[m][prec] = t;
+            if (!w.Lscr[m][prec]) TRY(dalloc(ctx, &t, 2 * (ninst - 1) * n));
+            if (!w.Lscr[m][prec]) w.Lscr[m][prec] = t;
+            return PF_OK;
+        };
+        if (prec == PF_FP64) TRY(make(static_cast<double *>(nullptr)));
+        else TRY(make(static_cast<float *>(nullptr)));
+        if (!w.LK[m]) TRY(dalloc(ctx, &w.LK[m], 8 * ninst));
+    }
+    return PF_OK;
+}
+
+// Storage that only a mapping by rule needs: where it does not fit, the run
+// takes the mapping that does without, and the batch does not ask again.
+bool fits(pf_ctx *ctx, pf_status &st) {
+    if (st != PF_ERR_OOM) return true;
+    cudaGetLastError();
+    ctx->ws.no_room = true;
+    st = PF_OK;
+    return false;
+}
+
 // Low-rank outages: Z and K of every outage instance of both matrices from
 // the base factors (after factor_both with lowrank).
 pf_status prepare_lowrank(pf_ctx *ctx, int prec, bool multi, cudaStream_t s) {
     Workspace &w = ctx->ws;
     const int ninst = ctx->dc.ninst;
-    const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
+    TRY(ensure_lowrank(ctx, prec));
     MultiLaunch zl;  // the solves for Z, several per block
     if (multi) {
         zl.K = multi_cases(ctx->dm, prec, 2 * (ninst - 1), ctx->num_sms, ctx->smem_optin, &zl.xs0);
@@ -2130,25 +2161,6 @@ pf_status prepare_lowrank(pf_ctx *ctx, int prec, bool multi, cudaStream_t s) {
     }
     for (int m = 0; m < 2; m++) {
         const DevMat &D = ctx->dm[m];
-        if (!w.LZ[m][prec]) {
-            const size_t nz = size_t(ninst) * 2 * size_t(std::max(1, D.n));
-            const size_t ns = size_t(2 * (ninst - 1)) * size_t(std::max(1, D.n));
-            if (prec == PF_FP64) {
-                double *z = nullptr, *g = nullptr;
-                TRY(dalloc(ctx, &z, nz));
-                TRY(dalloc(ctx, &g, ns));
-                w.LZ[m][prec] = z;
-                w.Lscr[m][prec] = g;
-            } else {
-                float *z = nullptr, *g = nullptr;
-                TRY(dalloc(ctx, &z, nz));
-                TRY(dalloc(ctx, &g, ns));
-                w.LZ[m][prec] = z;
-                w.Lscr[m][prec] = g;
-            }
-            (void)elt;
-        }
-        if (!w.LK[m]) TRY(dalloc(ctx, &w.LK[m], size_t(8) * size_t(ninst)));
         const void *F = prec == PF_FP64 ? (const void *)w.F64[m] : (const void *)w.F32[m];
         const void *TV = ctx->tune.tail != 2 ? w.TV[m][prec] : nullptr;
         cudaError_t e = counted(ctx, PF_K_SOLVE, 2, s, [&] {
@@ -2342,18 +2354,8 @@ bool cluster_applies(pf_ctx *ctx, const pf_run_opts *o) {
     return fdpf_cl_fits(ctx->cl_smem);
 }
 
-pf_status ensure_cluster(pf_ctx *ctx) {
-    if (ctx->cl[0].tasks) return PF_OK;
-    for (int w = 0; w < 2; w++) TRY(upload_cluster(ctx, w));
-    return PF_OK;
-}
-
-// Rebuilds the cluster engine's programs with g subtree levels per step:
-// the device copies are freed (uploaded again on the next use) and a CUDA
-// graph that launched the old ones is dropped.
-pf_status set_cluster_group(pf_ctx *ctx, int g) {
-    if (g == ctx->cl_group) return PF_OK;
-    drop_graph(ctx);
+// Frees the device copies of the cluster engine's programs.
+void free_cluster(pf_ctx *ctx) {
     for (int w = 0; w < 2; w++) {
         ClMat &M = ctx->cl[w];
         void *ptrs[] = {M.tpar, M.tcp, M.tcdep, M.tcpos, M.tdepth, M.vsrc, M.vals, M.tasks, M.tptr, M.steps,
@@ -2364,6 +2366,23 @@ pf_status set_cluster_group(pf_ctx *ctx, int g) {
         ctx->clW[w] = nullptr;
         M = ClMat();
     }
+}
+
+pf_status ensure_cluster(pf_ctx *ctx) {
+    if (ctx->cl[0].tasks) return PF_OK;
+    pf_status st = PF_OK;
+    for (int w = 0; w < 2 && st == PF_OK; w++) st = upload_cluster(ctx, w);
+    if (st != PF_OK) free_cluster(ctx);  // all of it or none
+    return st;
+}
+
+// Rebuilds the cluster engine's programs with g subtree levels per step:
+// the device copies are freed (uploaded again on the next use) and a CUDA
+// graph that launched the old ones is dropped.
+pf_status set_cluster_group(pf_ctx *ctx, int g) {
+    if (g == ctx->cl_group) return PF_OK;
+    drop_graph(ctx);
+    free_cluster(ctx);
     ctx->cl_group = g;
     for (int w = 0; w < 2; w++) TRY(build_cluster(ctx, w, ctx->hcl[w], g));
     ctx->cl_smem = cluster_smem_layout(ctx);
@@ -2830,20 +2849,32 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     MultiLaunch ml;
     const bool multi = (ctx->tune.tail == 0 || ctx->tune.tail == 3) &&
                        (ctx->tune.threads == 0 || ctx->tune.threads == 512) && ctx->tune.cluster <= 1 &&
-                       multi_refines(ctx, opts);
+                       multi_refines(ctx, opts) && !w.no_room;
     const bool by_rule = multi && ctx->tune.outage == 0 && ctx->dc.ninst > 1 && opts->flat_start &&
                          outages_connected(ctx);
     if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2 || by_rule))
-        TRY(ensure_multi(ctx, prec, opts->ir_max > 0, ctx->tune.cluster == 0 ? ctx->dc.ncase : 0, ctx->nbus, ml));
-    ctx->lowrank_by_rule = by_rule && ml.K > 0;
-    if (ctx->lowrank_by_rule) {
-        if (!w.own_now) {
-            TRY(dalloc(ctx, &w.own_now, size_t(ctx->dc.ncase)));
-            const cudaError_t e = cudaMemsetAsync(w.own_now, 0, sizeof(int) * size_t(ctx->dc.ncase), s);
+    {
+        pf_status st = ensure_multi(ctx, prec, opts->ir_max > 0, ctx->tune.cluster == 0 ? ctx->dc.ncase : 0, ctx->nbus, ml);
+        if (st == PF_OK && by_rule && ml.K > 0) st = ensure_lowrank(ctx, prec);
+        if (st == PF_OK && by_rule && ml.K > 0 && !w.own_now) {
+            st = dalloc(ctx, &w.own_now, size_t(ctx->dc.ncase));
+            const cudaError_t e =
+                st == PF_OK ? cudaMemsetAsync(w.own_now, 0, sizeof(int) * size_t(ctx->dc.ncase), s) : cudaSuccess;
             if (e != cudaSuccess) return cuda_fail(ctx, e, "outage marks");
         }
-        ml.own_now = w.own_now;
+        if (!fits(ctx, st)) {
+            ml = MultiLaunch();
+            drop_graph(ctx);  // it may use what is freed
+            if (by_rule)
+                for (int m = 0; m < 2; m++) {
+                    dfree(ctx, w.LZ[m][prec]); w.LZ[m][prec] = nullptr;
+                    dfree(ctx, w.Lscr[m][prec]); w.Lscr[m][prec] = nullptr;
+                }
+        }
+        TRY(st);
     }
+    ctx->lowrank_by_rule = by_rule && ml.K > 0;
+    if (ctx->lowrank_by_rule) ml.own_now = w.own_now;
     const bool lowrank = ctx->dc.ninst > 1 && (ctx->tune.outage == 2 || ctx->lowrank_by_rule);
     TRY(factor_both(ctx, prec, s, lowrank, false, ml.K > 0));
     if (lowrank) {
@@ -3083,7 +3114,12 @@ pf_status run_once(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, double 
     const pf_tuning &tn = ctx->tune;
     const int by_rule = tn.cluster == 0 && tn.tail == 0 && tn.threads == 0 ? PF_ENGINE_CLUSTER : PF_ENGINE_BLOCK;
     const int want = opts->engine != PF_ENGINE_AUTO ? opts->engine : tn.engine != 0 ? tn.engine : by_rule;
-    const bool use_cluster = want == PF_ENGINE_CLUSTER && cluster_applies(ctx, opts);
+    bool use_cluster = want == PF_ENGINE_CLUSTER && cluster_applies(ctx, opts);
+    if (use_cluster && opts->engine == PF_ENGINE_AUTO && tn.engine == 0) {  // by rule
+        pf_status st = w.no_room ? PF_ERR_OOM : ensure_cluster(ctx);
+        use_cluster = fits(ctx, st);
+        TRY(st);
+    }
     const int engine = use_cluster ? PF_ENGINE_CLUSTER
                                    : (want == PF_ENGINE_LANES && lanes_ok ? PF_ENGINE_LANES : PF_ENGINE_BLOCK);
     if (engine == PF_ENGINE_LANES) {
@@ -3505,8 +3541,10 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
         // more grids than SMs: k_fdpf_pack keeps two grids on an SM, where
         // this kernel's registers allow one (256 grids of 2,000 to 80,000 buses,
         // FP32: 149 ms against 184; 100 grids 133 ms here, 137 there)
-        if (ngrid <= ctx->num_sms && (ctx->tune.tail == 0 || ctx->tune.tail == 3) && multi_refines(ctx, opts)) {
+        if (ngrid <= ctx->num_sms && (ctx->tune.tail == 0 || ctx->tune.tail == 3) && multi_refines(ctx, opts) &&
+            !w.no_room) {
             st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, p.ml);
+            if (!fits(ctx, st)) p.ml = MultiLaunch();
             if (st != PF_OK) return pack_fail(pk, st, "grid %d: %s", g, ctx->err.c_str());
         }
         p.A0 = w.A[0];

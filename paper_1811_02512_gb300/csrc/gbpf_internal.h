@@ -468,6 +468,7 @@ struct Workspace {
     std::vector<int> own_case;
     std::vector<unsigned char> own_key;  // those arguments (run_device_work), empty: loads changed
     int ninst_full = 0;       // instances that the factor storage is for
+    bool no_room = false;     // storage that a mapping by rule wanted did not fit: not asked for again
     int2 *mx = nullptr;       // [ncase][nbus] its refined solutions (FP32)
     void *mxg = nullptr;      // [ncase][rows in global memory] of 8 bytes
     size_t mxg_count = 0;

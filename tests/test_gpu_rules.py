@@ -75,3 +75,37 @@ def test_outages_that_fail(bad, fallback, prec):
     assert _launches(g, gbpf.PF_K_RUN) == 1
     g.close()
     own.close()
+
+
+# With no memory left for what only a mapping by rule needs, the run takes the
+# mapping that does without.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_no_room_for_the_mapping_by_rule(prec):
+    case = gridgen.delaunay_raw(3000, 21).scaled_network(1.0 / 64)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    cut = set(gridgen.bridges(case.n, case.f, case.t, case.status))
+    out = np.array([k for k in range(case.m) if k not in cut][:600], np.int32)
+    ncase = len(out)
+    g = gbpf.Grid(case)
+    g.set_cases(ncase, None, out)
+    gbpf.pf_set_tuning(g.ctx, outage=1)
+    st1, res1, vm1, va1 = _run(g, case.n, ncase, p, tol=1e-8)  # storage of the own factors
+    gbpf.pf_set_tuning(g.ctx)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    vm = torch.zeros((ncase, case.n), dtype=torch.float64, device="cuda")
+    va = torch.zeros_like(vm)
+    torch.cuda.synchronize()
+    # the low-rank storage is 57 MB at least (FP32; 115 MB in FP64)
+    take = torch.cuda.mem_get_info()[0] - (32 << 20)
+    hold = torch.empty(take, dtype=torch.uint8, device="cuda")
+    try:
+        for _ in range(3):
+            st, res = gbpf.pf_run_to_tol(g.ctx, gbpf.run_opts(gbpf.PF_FDPF, p, tol=1e-8), vm, va, ncase)
+            assert st == st1 == gbpf.PF_OK, gbpf.pf_last_error(g.ctx)
+            assert np.array_equal(res["iters"], res1["iters"])
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(vm.cpu().numpy(), vm1) and np.array_equal(va.cpu().numpy(), va1)
+    g.close()
