@@ -824,7 +824,7 @@ def main():
     engine_used = (tuning or {}).get("engine", engine)
     tn = tuning or {}
     # the several-cases-per-block kernel runs what the base factor can solve
-    multi = (tn.get("tail", 0) in (0, 3) and tn.get("threads", 0) in (0, 512) and tn.get("cluster", 0) <= 1
+    multi = (tn.get("tail", 0) in (0, 3) and tn.get("threads", 0) in (0, 512)
              and (outage is None or tn.get("outage", 0) != 1))
     kname = "k_fdpf_cl" if engine_used == gbpf.PF_ENGINE_CLUSTER else "k_fdpf_multi" if multi else "k_fdpf"
     hbm["traffic"] = measured_traffic(args.workload, prec_name, ncase, kname) if method == gbpf.PF_FDPF else None

@@ -157,7 +157,9 @@ enum { PF_ENGINE_AUTO = 0, PF_ENGINE_BLOCK = 1, PF_ENGINE_LANES = 2, PF_ENGINE_C
  *            W^T D_T^-1 z_T: two parallel gathers instead of a level chain;
  *            W formed after every factorisation; block engine runs whose
  *            solves all use the base factor: one instance, or low-rank
- *            outages -- other runs use form 1);
+ *            outages -- other runs use form 1; with block size 0 or 512 these
+ *            are the runs of several cases per block, or of the cluster size
+ *            asked for);
  *   outage   1: every single-branch outage case has its own B'/B'' factors,
  *            2: outage cases reuse the base factors with a low-rank
  *            (Woodbury) correction of each solve by the outaged branch's

@@ -230,11 +230,11 @@ size_t multi_smem_bytes(const MultiLaunch &ml, const DevMat *m, int prec) {
 // 0.57 on 1,000 buses, 0.88 against 0.85 on 2,000, 1.08 against 1.18 on 3,000,
 // 1.92 against 2.66 on 10,000, 7.1 against 10.9 on 40,000; FP64 8.6 against
 // 12.3 on 40,000; nine cases of 10,000 buses 2.05 against 2.66).
-int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem) {
+int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem, int most) {
     constexpr int kMultiClBuses = 2500;
-    if (nbus < kMultiClBuses) return 1;
+    if (most == 0 && nbus < kMultiClBuses) return 1;
     for (int C : {16, 8})
-        if (groups * C <= num_sms &&
+        if ((most == 0 || C <= most) && groups * C <= num_sms &&
             (prec == PF_FP64 ? multi_clusters_f64(C, smem) : multi_clusters_f32(C, smem)) >= groups)
             return C;
     return 1;

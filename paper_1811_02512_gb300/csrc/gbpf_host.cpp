@@ -2079,8 +2079,8 @@ bool multi_refines(const pf_ctx *ctx, const pf_run_opts *o) {
 }
 
 // The several-cases-per-block launch of this batch: its shape and storage (K
-// = 0: it does not apply); groups, nbus: see multi_cluster_size (0: no clusters).
-pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus, MultiLaunch &ml) {
+// = 0: it does not apply); groups, nbus, most: see multi_cluster_size (most 1: no clusters).
+pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus, int most, MultiLaunch &ml) {
     Workspace &w = ctx->ws;
     ml.K = multi_cases(ctx->dm, prec, ctx->dc.ncase, ctx->num_sms, ctx->smem_optin, &ml.xs0);
     if (ml.K == 0) return PF_OK;
@@ -2093,7 +2093,7 @@ pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus,
         ml.K = 0;
         return PF_OK;
     }
-    if (ml.K == 1 && groups > 0) ml.C = multi_cluster_size(groups, nbus, ctx->num_sms, prec, smem);
+    if (ml.K == 1 && most != 1) ml.C = multi_cluster_size(groups, nbus, ctx->num_sms, prec, smem, most);
     if (!w.redo) TRY(dalloc(ctx, &w.redo, size_t(ctx->dc.ncase)));
     ml.redo = w.redo;
     const size_t rows = size_t(ctx->dc.ncase) * size_t(ml.C > 1 ? std::max(ctx->dm[0].n, ctx->dm[1].n) : ml.xs0);
@@ -2839,7 +2839,8 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
         return PF_OK;
     }
     // several cases per block, wherever all solves use the base factor and the
-    // tuning names no other tail form, block size or cluster: faster than
+    // tuning names no other tail form or block size (a cluster size there is
+    // this kernel's): faster than
     // k_fdpf at every size tried, its 16-block cluster for one case included
     // (FP32, ir_tol 1e-3: 0.27 ms against 0.55 on 200 buses, 0.87 against 1.35
     // on 2,643, 4.8 against 11.5 on 40,000; FP64 0.38 against 0.54, 8.6
@@ -2848,13 +2849,13 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
     // 1,425-bus grid: their own factors alone took 2.3 ms).
     MultiLaunch ml;
     const bool multi = (ctx->tune.tail == 0 || ctx->tune.tail == 3) &&
-                       (ctx->tune.threads == 0 || ctx->tune.threads == 512) && ctx->tune.cluster <= 1 &&
-                       multi_refines(ctx, opts) && !w.no_room;
+                       (ctx->tune.threads == 0 || ctx->tune.threads == 512) && multi_refines(ctx, opts) && !w.no_room;
+    const int asked = ctx->tune.engine == PF_ENGINE_CLUSTER ? 0 : ctx->tune.cluster;  // there: levels per step
     const bool by_rule = multi && ctx->tune.outage == 0 && ctx->dc.ninst > 1 && opts->flat_start &&
                          outages_connected(ctx);
     if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2 || by_rule))
     {
-        pf_status st = ensure_multi(ctx, prec, opts->ir_max > 0, ctx->tune.cluster == 0 ? ctx->dc.ncase : 0, ctx->nbus, ml);
+        pf_status st = ensure_multi(ctx, prec, opts->ir_max > 0, ctx->dc.ncase, ctx->nbus, asked, ml);
         if (st == PF_OK && by_rule && ml.K > 0) st = ensure_lowrank(ctx, prec);
         if (st == PF_OK && by_rule && ml.K > 0 && !w.own_now) {
             st = dalloc(ctx, &w.own_now, size_t(ctx->dc.ncase));
@@ -3345,7 +3346,15 @@ pf_status pf_autotune(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doub
     if (std::max(ctx->hm[0].max_col, ctx->hm[1].max_col) <= kDepMaxCol) factors.push_back(1);
     std::vector<int> tails{2};
     if (o.method == PF_FDPF && (ctx->dm[0].npf2 > 0 || ctx->dm[1].npf2 > 0)) tails.push_back(1);
-    if (o.method == PF_FDPF && (ctx->dm[0].npf3 > 0 || ctx->dm[1].npf3 > 0)) tails.push_back(3);
+    // form 3 is also what runs the several-cases-per-block kernel, on grids
+    // without the inverse too: what an untuned run takes is among the
+    // candidates (an FP32 case of 10,000 buses, 3.25 ms, was tuned to 4.53,
+    // one of 40,000, 6.3 ms, to 9.7 while cluster sizes meant k_fdpf's only)
+    int rows_g = 0;
+    if (o.method == PF_FDPF && (ctx->dm[0].npf3 > 0 || ctx->dm[1].npf3 > 0 ||
+                                (multi_refines(ctx, &o) &&
+                                 multi_cases(ctx->dm, prec, ncase, ctx->num_sms, ctx->smem_optin, &rows_g) > 0)))
+        tails.push_back(3);
     std::vector<int> outages{1};
     if (o.method == PF_FDPF && ctx->dc.ninst > 1) outages.push_back(2);
     // the lane engine has no cluster, tail or outage choice; the cluster
@@ -3543,7 +3552,7 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
         // FP32: 149 ms against 184; 100 grids 133 ms here, 137 there)
         if (ngrid <= ctx->num_sms && (ctx->tune.tail == 0 || ctx->tune.tail == 3) && multi_refines(ctx, opts) &&
             !w.no_room) {
-            st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, p.ml);
+            st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, 0, p.ml);
             if (!fits(ctx, st)) p.ml = MultiLaunch();
             if (st != PF_OK) return pack_fail(pk, st, "grid %d: %s", g, ctx->err.c_str());
         }

@@ -643,8 +643,9 @@ struct NrLaunch;
 // many as fit shared memory at most; 0 where not even one does.
 int multi_cases(const DevMat *m, int prec, int ncase, int num_sms, size_t smem_optin, int *xs0);
 // Blocks per case for `groups` cases (or grids of a pack, the largest of nbus
-// buses) of one case per block each with `smem` bytes: 16, 8 or 1.
-int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem);
+// buses) of one case per block each with `smem` bytes: 16, 8 or 1; most: 16 or
+// 8 asked for, 0 by size.
+int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem, int most = 0);
 // The columns of Z of launch_lowrank, ml.K of them per block on instance 0's
 // factor with its top's inverse; z_done there.
 cudaError_t launch_lowrank_z_multi(const MultiLaunch &ml, const DevNet &dn, const DevCases &dc, const DevMat *m, int which,

@@ -109,3 +109,58 @@ def test_no_room_for_the_mapping_by_rule(prec):
         torch.cuda.empty_cache()
     assert np.array_equal(vm.cpu().numpy(), vm1) and np.array_equal(va.cpu().numpy(), va1)
     g.close()
+
+
+# What an untuned run takes can be set by hand and is among the tuner's
+# candidates: the same bits from the mapping by rule and from its fields.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("n,ncase,cluster", [(3000, 1, 16), (3000, 12, 8), (900, 1, 1)])
+def test_tuning_reaches_the_mapping_by_rule(n, ncase, cluster, prec):
+    case = gridgen.delaunay_raw(n, 7).scaled_network(1.0 / 64)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    sc = gridgen.scenarios(case, n_load=ncase, n_outage=0, seed=3)
+    g = gbpf.Grid(case)
+    g.set_cases(ncase, sc.load_scale, sc.outage)
+    out = []
+    for tuning in (dict(engine=gbpf.PF_ENGINE_BLOCK),
+                   dict(engine=gbpf.PF_ENGINE_BLOCK, cluster=cluster, factor=1, tail=3, outage=1)):
+        gbpf.pf_set_tuning(g.ctx, **tuning)
+        out.append(_run(g, n, ncase, p, tol=1e-8))
+    assert out[0][0] == gbpf.PF_OK and np.array_equal(out[0][1], out[1][1])
+    assert np.array_equal(out[0][2], out[1][2]) and np.array_equal(out[0][3], out[1][3])
+    # asked for where the size would not have it: as many blocks, the same states to rounding
+    if cluster == 1:
+        gbpf.pf_set_tuning(g.ctx, engine=gbpf.PF_ENGINE_BLOCK, cluster=16, tail=3)
+        st, res, vm, va = _run(g, n, ncase, p, tol=1e-8)
+        assert st == gbpf.PF_OK and res["iters"][0] == out[0][1]["iters"][0]
+        assert np.abs(vm - out[0][2]).max() <= 1e-9 and np.abs(va - out[0][3]).max() <= 1e-9
+    g.close()
+
+
+# A star has one level and no narrow top: the tuner tries form 3 there too.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_tuner_on_a_grid_without_a_top(prec):
+    m = 400
+    z = np.zeros(m + 1)
+    case = gridgen.Case("star", np.array([gridgen.SLACK] + [gridgen.PQ] * m, np.int32),
+                        np.r_[0.0, np.linspace(0.01, 0.1, m)], np.r_[0.0, np.full(m, 0.01)], z.copy(), z.copy(), z.copy(),
+                        np.ones(m + 1), z.copy(), np.zeros(m, np.int32), np.arange(1, m + 1, dtype=np.int32),
+                        np.full(m, 0.01), np.full(m, 0.05), np.zeros(m), np.zeros(m), np.ones(m, np.int32))
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    g = gbpf.Grid(case)
+    g.set_cases(40)
+    vm = torch.zeros((40, m + 1), dtype=torch.float64, device="cuda")
+    va = torch.zeros_like(vm)
+    _launches(g, gbpf.PF_K_RUN)
+    t = gbpf.pf_autotune(g.ctx, gbpf.run_opts(gbpf.PF_FDPF, p, tol=1e-8), vm, va, reps=1)
+    runs = _launches(g, gbpf.PF_K_RUN)
+    assert t["tail"] in (2, 3) or t["engine"] == gbpf.PF_ENGINE_LANES
+    # one block per case, two factor forms, three block sizes, tail 2 and 3,
+    # each once untimed and once timed (the lane engine counts more launches)
+    assert runs >= 2 * 2 * 3 * 2
+    gbpf.pf_set_tuning(g.ctx, engine=gbpf.PF_ENGINE_BLOCK, cluster=1, factor=1, tail=3, outage=1, threads=512)
+    st, res, vm1, va1 = _run(g, m + 1, 40, p, tol=1e-8)
+    gbpf.pf_set_tuning(g.ctx, engine=gbpf.PF_ENGINE_BLOCK)
+    st0, res0, vm0, va0 = _run(g, m + 1, 40, p, tol=1e-8)
+    assert st == st0 == gbpf.PF_OK and np.array_equal(vm0, vm1) and np.array_equal(va0, va1)
+    g.close()
