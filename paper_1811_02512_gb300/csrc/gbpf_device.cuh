@@ -985,12 +985,22 @@ __device__ __forceinline__ bool fx_va_ok(double t) {
     return (unsigned(__double2hiint(t)) & 0x7fffffffu) < 0x401f0000u;
 }
 
-// e + jf rotated by d (units 2^-60, |d| <= 0.2); every lane of the warp that
-// is here takes the short series when all can.
+// e + jf rotated by d (units 2^-60, |d| <= 0.2); the lanes of a case that are
+// here (every K-th of the warp) take the short series when all of them can: a
+// case's bits then do not depend on the other cases of its warp.  (A choice
+// per lane made the one-case kernels 7 % slower.)
+template <int K>
 __device__ __forceinline__ int4 fx_rotate(const int4 &v, long long d) {
     long long sd, cm;
-    const bool small = (d < 0 ? -d : d) < (1ll << 50);
-    fx_small_sincos(d, __all_sync(__activemask(), small), sd, cm);
+    bool small = (d < 0 ? -d : d) < (1ll << 50);
+    const unsigned here = __activemask();
+    if constexpr (K == 1) {
+        small = __all_sync(here, small);
+    } else {
+        constexpr unsigned mine = K == 2 ? 0x55555555u : 0x11111111u;
+        small = ((__ballot_sync(here, !small) >> (threadIdx.x % K)) & mine) == 0u;
+    }
+    fx_small_sincos(d, small, sd, cm);
     const FxLimbs s = fx_split(sd), c = fx_split(cm);
     FxAcc a{0, 0}, b{0, 0};
     fx_mac(a, v.x, v.y, c.h, c.l);
@@ -1038,7 +1048,7 @@ __device__ __forceinline__ int4 fx_polar_any(double vm, double va) {
 __device__ __forceinline__ bool fx_angle_step(int4 *ef, double d, double vm, double va) {
     const unsigned h = unsigned(__double2hiint(d)) & 0x7fffffffu;
     if (h < 0x3fc99999u) {  // |d| < 0.2
-        *ef = fx_rotate(*ef, fx_from_double(d, 60));
+        *ef = fx_rotate<1>(*ef, fx_from_double(d, 60));
         return !fx_va_ok(va);
     }
     if (!fx_va_ok(va)) return true;

@@ -793,7 +793,7 @@ __device__ __forceinline__ void update_multi(const MultiArgs &ma, MultiShared<K>
             const long long t = s0 + d;
             st.th[at] = t;
             if (ad < 230584300921369395ull)  // 0.2
-                st.ef[at] = fx_rotate(v, d);
+                st.ef[at] = fx_rotate<K>(v, d);
             else
                 st.ef[at] = fx_polar60(st.vv[at], t);
         } else {
@@ -987,7 +987,8 @@ __global__ void __launch_bounds__(kMultiThreads, 1) k_fdpf_multi(const __grid_co
 // One case per cluster of ma.C blocks: the nodal work -- mismatch, residual,
 // update, three quarters of an iteration on one block -- over all of them, the
 // sweeps on the first, whose level chain bounds it then.  The sums are those of
-// one block, so the iterates are the same.  One FP32 case of 40,000 buses,
+// one block; the iterates may differ in the last bits (fx_rotate's choice by
+// warp).  One FP32 case of 40,000 buses,
 // refined to 1e-10, factors included: 10.9 ms on one block, 7.1 on 16.
 template <class T>
 __global__ void __launch_bounds__(kMultiThreads, 1) k_fdpf_multi_cl(const __grid_constant__ MultiArgs ma) {

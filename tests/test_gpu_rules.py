@@ -164,3 +164,26 @@ def test_tuner_on_a_grid_without_a_top(prec):
     st0, res0, vm0, va0 = _run(g, m + 1, 40, p, tol=1e-8)
     assert st == st0 == gbpf.PF_OK and np.array_equal(vm0, vm1) and np.array_equal(va0, va1)
     g.close()
+
+
+# A case's result is its own: the same bits whatever other cases the batch
+# holds (2 and 4 cases to a block).
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("ncase", [201, 307])
+def test_bits_do_not_depend_on_the_other_cases(ncase, prec):
+    case = gridgen.delaunay_raw(700, 5).scaled_network(1.0 / 32)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    # every eighth case stays, the others take other loads (some too heavy ones)
+    out = []
+    for k in range(4):
+        ls = np.random.default_rng(2).normal(1.0, 0.08, (ncase, case.n))
+        rest = np.arange(ncase) % 8 != 0
+        ls[rest] *= np.random.default_rng(10 + k).uniform(0.3, 1.3, (int(rest.sum()), 1))
+        g = gbpf.Grid(case)
+        g.set_cases(ncase, ls)
+        st, res, vm, va = _run(g, case.n, ncase, p, tol=1e-10)
+        assert np.all(res["status"][::8] == gbpf.PF_OK)
+        out.append((res["iters"][::8], vm[::8], va[::8]))
+        g.close()
+    for its, vm, va in out[1:]:
+        assert np.array_equal(its, out[0][0]) and np.array_equal(vm, out[0][1]) and np.array_equal(va, out[0][2])
