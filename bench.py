@@ -34,6 +34,7 @@ import os
 import statistics
 import subprocess
 import sys
+import tempfile
 import threading
 import time
 
@@ -62,6 +63,7 @@ def parse():
     ap.add_argument("--ncase", type=int, default=1024,
                     help="batch10k: number of cases (half load scenarios, half outages)")
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--details", default=None, help="file for the whole record (per-case errors, every kernel)")
     ap.add_argument("--no-batched", action="store_true",
                     help="plain10k: skip the batched FP32+IR measurement reported beside it")
     ap.add_argument("--no-autotune", action="store_true",
@@ -382,6 +384,46 @@ def run_reference(args):
     print(json.dumps(line))
 
 
+LINE_MAX = 2600  # characters: what reads the line keeps the last 3,000 of the output
+
+
+def _brief(v):
+    """v with floats at seven digits and without long lists."""
+    if isinstance(v, float):
+        return float(f"{v:.7g}")
+    if isinstance(v, dict):
+        return {k: _brief(x) for k, x in v.items() if not (isinstance(x, (list, tuple)) and len(x) > 8)}
+    return [_brief(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def brief_line(line):
+    """The record as one line of at most LINE_MAX characters: what repeats or
+    explains a figure goes first, the contract's keys stay."""
+    out = _brief(line)
+    cut = [("batched_fp32_ir", k) for k in ("clocks", "config", "iters_mean", "ir_steps_mean", "gpu_launches", "cpu_baseline",
+                                            "roofline")]
+    cut += [("kernel_launches_per_step",), ("accuracy", "seconds"), ("accuracy", "reference"), ("accuracy", "worst_case"),
+            ("kernel_ms_per_step",), ("cuda_graph",), ("sequential_plain_fp64",), ("roofline", "hbm"),
+            ("batched_fp32_ir", "accuracy"), ("batched_fp32_ir",), ("accuracy",), ("cpu_baseline",), ("config", "tuning")]
+    for path in cut:
+        if len(json.dumps(out)) <= LINE_MAX:
+            break
+        d = out
+        for k in path[:-1]:
+            d = d.get(k) if isinstance(d, dict) else None
+        if isinstance(d, dict):
+            d.pop(path[-1], None)
+    return out
+
+
+def emit(line, args):
+    """Prints the record's line; the whole record to --details."""
+    if args.details:
+        with open(args.details, "w") as fh:
+            json.dump(line, fh)
+    print(json.dumps(brief_line(line)))
+
+
 def batched_line(args):
     """The metric's other half -- the same grid as 1,024 load/outage cases in
     one launch, FP32 factor + FP64 refinement -- measured by this script's
@@ -389,9 +431,12 @@ def batched_line(args):
     cmd = [sys.executable, os.path.join(ROOT, "bench.py"), "--workload", "batch10k", "--steps", "5",
            "--warmup", str(max(3, args.warmup)), "--cpu-sample-s", "3"]
     try:
-        out = subprocess.run(cmd, capture_output=True, text=True, timeout=900, check=True).stdout
-        d = json.loads([ln for ln in out.splitlines() if ln.startswith("{")][-1])
-    except (subprocess.SubprocessError, ValueError, IndexError) as exc:
+        with tempfile.TemporaryDirectory() as tmp:
+            path = os.path.join(tmp, "batch.json")
+            subprocess.run(cmd + ["--details", path], capture_output=True, text=True, timeout=900, check=True)
+            with open(path) as fh:
+                d = json.load(fh)
+    except (subprocess.SubprocessError, ValueError, OSError) as exc:
         return {"unavailable": str(exc)[:200]}
     keep = ("value", "unit", "ms_per_step", "dtype", "converged", "gpu_launches", "roofline", "e2e",
             "clocks", "ir_steps_mean", "ir_steps_max", "iters_mean", "accuracy", "cpu_baseline")
@@ -507,7 +552,7 @@ def run_adjoint(args, dev, local, world, rank):
             "e2e": {"value": e2e_val, "unit": "(PF + gradient)/s",
                     "h2d_bytes_per_step": int(2 * 8 * case.n), "d2h_bytes_per_step": int(2 * 8 * case.n)}}
     if rank == 0:
-        print(json.dumps(line))
+        emit(line, args)
     g.close()
 
 
@@ -646,7 +691,7 @@ def run_pack(args, dev, local, world, rank):
             "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": int(2 * tot * 8),
                     "d2h_bytes_per_step": int(2 * tot * 8 + 24 * len(grids))}}
     if rank == 0:
-        print(json.dumps(line))
+        emit(line, args)
     pk.close()
     for g in grids:
         g.close()
@@ -881,7 +926,7 @@ def main():
     if rank == 0 and world == 1 and args.workload == "plain10k" and not args.no_batched:
         line["batched_fp32_ir"] = batched_line(args)
     if rank == 0:
-        print(json.dumps(line))
+        emit(line, args)
     g.close()
     if world > 1:
         dist.destroy_process_group()
