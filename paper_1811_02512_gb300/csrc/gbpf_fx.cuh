@@ -233,8 +233,8 @@ GBPF_FX long long fx_recip(long long v) {
            ((static_cast<long long>(y) * cl) >> 26);
 }
 
-// sin d and 1 - cos d in units 2^-60 for d in units 2^-60, |d| <= 0.2.
-// small: |d| < 2^-10.
+// sin d and 1 - cos d in units 2^-60 for d in units 2^-60, |d| <= 0.2, within
+// 2.5 and 1 units.  small: |d| < 2^-10.
 GBPF_FX void fx_small_sincos(long long d, bool small, long long &sd, long long &cm) {
     const unsigned long long x = static_cast<unsigned long long>(d < 0 ? -d : d) << 4;  // 0.64
     unsigned long long s, c;
