@@ -423,8 +423,8 @@ __device__ double cl_mismatch(const ClRun &a, int rank, int which, const uint32_
     return cl_exchange_max<C>(mx, which, red, mkey, kbase);
 }
 
-// The fixed-point form (as k_fdpf's cluster_mismatch_fx): left = this thread
-// saw a bus leave the fixed-point range; the maximum is then the all-ones key.
+// The fixed-point form: left = this thread saw a bus leave the fixed-point
+// range; the maximum is then the all-ones key.
 template <int C>
 __device__ double cl_mismatch_fx(const ClRun &a, int rank, int which, const uint32_t *xbase, double *red,
                                  unsigned long long *mkey, const uint32_t *kbase, bool full, bool left) {

@@ -1435,7 +1435,6 @@ pf_status upload_matrix(pf_ctx *ctx, const HostMat &H, DevMat &D) {
     D.t0 = H.t0;
     D.nt = H.nt;
     D.ntl = H.ntl;
-    TRY(upload_padded(ctx, &D.trange, std::vector<int>{H.t0, H.n}));
     D.npf2 = int(H.pf2.size());
     D.npb2 = int(H.pb2.size());
     D.npf3 = D.npb3 = 0;

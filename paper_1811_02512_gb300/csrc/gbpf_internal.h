@@ -82,7 +82,6 @@ struct DevMat {
     // into [tv_f: forward slots | tv_b: backward slots | tv_p: entries below
     // t0] from the value slots TVsrc (-1: zero).
     int t0 = 0, nt = 0, ntl = 0;
-    int *trange = nullptr;     // {t0, n}
     int npf2 = 0, npb2 = 0;
     Piece *pf2 = nullptr, *pb2 = nullptr;
     int *SKf = nullptr, *SIf = nullptr, *SKb = nullptr, *SIb = nullptr;

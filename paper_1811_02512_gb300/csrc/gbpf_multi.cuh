@@ -106,10 +106,10 @@ __device__ __forceinline__ void sync_multi() {
 // ranges two steps before it -- so that a level costs its gathers from shared
 // memory and one memory latency at most.  (Staged through shared memory by
 // bulk copies, 8 KB at a time and four in flight, the copies' latency bound
-// the sweeps: 55 us for a sweep of B' of 10,000 buses, 4 cases.)
-// More warps only add a step's fixed instructions, and at 64 registers spills
-// that the small L1 beside the solve vectors does not hold: 34 us a sweep with
-// 1,024 threads, 22 with 512.
+// the sweeps: 56 us forward and 47 backward for B' of 10,000 buses, 4 FP32
+// cases, by clock stamps; 32 and 41 this way.)  512 threads: more warps add a
+// step's fixed instructions, and at 64 registers spills that the small L1
+// beside the solve vectors does not hold.
 template <class T, int K, int XG>
 __device__ __noinline__ void sweep_multi(const int2 *steps, int ns, const int *ptr, const int *idx, const T *val,
                                          const T *dinv, XVec<T, K, XG> x) {
