@@ -340,6 +340,22 @@ cudaError_t launch_fdpf(const DevNet &dn, const DevCases &dc, const DevMat *m, i
                            : fdpf_run_f32(a, smem, cluster, threads, s);
 }
 
+// Rows of one case's solve vector that may lie in global memory: those below
+// the narrow top, and at most half of them all.
+static bool multi_rows_out(const DevMat *m, long long x) {
+    const int nmax = m[0].n > m[1].n ? m[0].n : m[1].n;
+    return x <= m[0].n - m[0].nt && x <= m[1].n && 2 * x <= nmax;
+}
+
+bool multi_fit(MultiLaunch &ml, const DevMat *m, int prec, size_t room) {
+    const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float), need = multi_smem_bytes(ml, m, prec);
+    if (need <= room) return true;
+    const long long x = ml.xs0 + (long long)((need - room) / elt) + 8;  // the sizes are rounded up
+    if (ml.K != 1 || !multi_rows_out(m, x)) return false;
+    ml.xs0 = int(x);
+    return multi_smem_bytes(ml, m, prec) <= room;
+}
+
 int multi_cases(const DevMat *m, int prec, int ncase, int num_sms, size_t smem_optin, int *xs0) {
     const size_t elt = prec == PF_FP64 ? sizeof(double) : sizeof(float);
     const int nmax = m[0].n > m[1].n ? m[0].n : m[1].n;
@@ -350,10 +366,8 @@ int multi_cases(const DevMat *m, int prec, int ncase, int num_sms, size_t smem_o
     // elements of the solve vectors and the top's vector that fit
     const long long cap = (long long)((smem_optin - 2048 - kMultiStepBytes) / elt) - 4;
     if (nmax + nt > cap) {
-        // one case, with rows below the narrow top (and at most half of
-        // them all) in global memory
-        const long long x = nmax + nt - cap;
-        if (x > m[0].n - m[0].nt || x > m[1].n || 2 * x > nmax) return 0;
+        const long long x = nmax + nt - cap;  // one case, with rows in global memory
+        if (!multi_rows_out(m, x)) return 0;
         *xs0 = int(x);
         return 1;
     }

@@ -2078,8 +2078,10 @@ bool multi_refines(const pf_ctx *ctx, const pf_run_opts *o) {
 }
 
 // The several-cases-per-block launch of this batch: its shape and storage (K
-// = 0: it does not apply); groups, nbus, most: see multi_cluster_size (most 1: no clusters).
-pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus, int most, MultiLaunch &ml) {
+// = 0: it does not apply); groups, nbus, most: see multi_cluster_size (most 1: no
+// clusters); fixed: static shared memory beyond 1 KB.
+pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus, int most, size_t fixed,
+                       MultiLaunch &ml) {
     Workspace &w = ctx->ws;
     ml.K = multi_cases(ctx->dm, prec, ctx->dc.ncase, ctx->num_sms, ctx->smem_optin, &ml.xs0);
     if (ml.K == 0) return PF_OK;
@@ -2087,11 +2089,14 @@ pf_status ensure_multi(pf_ctx *ctx, int prec, bool refine, int groups, int nbus,
     ml.net = ctx->mnet;
     for (int q = 0; q < 2; q++)
         TRY(ensure_multi_steps(ctx, q, prec, ml.K, ctx->dm[q].npf3 > 0, ml.steps[q]));
-    const size_t smem = multi_smem_bytes(ml, ctx->dm, prec);
-    if (smem + 1024 > ctx->smem_optin) {  // a grid of very many levels: its steps do not fit
+    // the steps of a grid of many levels may take more than multi_cases left
+    // them (a pack's grid of 68,000 buses: 100 bytes, and k_fdpf_pack's 61 ms
+    // instead of 17)
+    if (!multi_fit(ml, ctx->dm, prec, ctx->smem_optin - 1024 - fixed)) {
         ml.K = 0;
         return PF_OK;
     }
+    const size_t smem = multi_smem_bytes(ml, ctx->dm, prec);
     if (ml.K == 1 && most != 1) ml.C = multi_cluster_size(groups, nbus, ctx->num_sms, prec, smem, most);
     if (!w.redo) TRY(dalloc(ctx, &w.redo, size_t(ctx->dc.ncase)));
     ml.redo = w.redo;
@@ -2854,7 +2859,7 @@ pf_status issue_fdpf(pf_ctx *ctx, const pf_run_opts *opts, double *vm_dev, doubl
                          outages_connected(ctx);
     if (multi && (ctx->dc.ninst == 1 || ctx->tune.outage == 2 || by_rule))
     {
-        pf_status st = ensure_multi(ctx, prec, opts->ir_max > 0, ctx->dc.ncase, ctx->nbus, asked, ml);
+        pf_status st = ensure_multi(ctx, prec, opts->ir_max > 0, ctx->dc.ncase, ctx->nbus, asked, 0, ml);
         if (st == PF_OK && by_rule && ml.K > 0) st = ensure_lowrank(ctx, prec);
         if (st == PF_OK && by_rule && ml.K > 0 && !w.own_now) {
             st = dalloc(ctx, &w.own_now, size_t(ctx->dc.ncase));
@@ -3551,7 +3556,7 @@ pf_status pf_pack_run(pf_pack *pk, const pf_run_opts *opts, double *vm_dev, doub
         // FP32: 149 ms against 184; 100 grids 133 ms here, 137 there)
         if (ngrid <= ctx->num_sms && (ctx->tune.tail == 0 || ctx->tune.tail == 3) && multi_refines(ctx, opts) &&
             !w.no_room) {
-            st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, 0, p.ml);
+            st = ensure_multi(ctx, prec, opts->ir_max > 0, ngrid, largest, 0, multi_args_bytes(), p.ml);
             if (!fits(ctx, st)) p.ml = MultiLaunch();
             if (st != PF_OK) return pack_fail(pk, st, "grid %d: %s", g, ctx->err.c_str());
         }

@@ -649,6 +649,9 @@ int multi_cluster_size(int groups, int nbus, int num_sms, int prec, size_t smem,
 // factor with its top's inverse; z_done there.
 cudaError_t launch_lowrank_z_multi(const MultiLaunch &ml, const DevNet &dn, const DevCases &dc, const DevMat *m, int which,
                                    int prec, const void *F, const void *TV, const void *TW, void *Z, cudaStream_t s);
+// Fits the launch to `room` bytes of dynamic shared memory: a single case's
+// solve vector gives up rows to global memory; false where that does not do.
+bool multi_fit(MultiLaunch &ml, const DevMat *m, int prec, size_t room);
 // Dynamic shared memory of the launch.
 size_t multi_smem_bytes(const MultiLaunch &ml, const DevMat *m, int prec);
 // fb (optional): the Newton-Raphson launch that unconverged cases fall back

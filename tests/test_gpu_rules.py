@@ -187,3 +187,37 @@ def test_bits_do_not_depend_on_the_other_cases(ncase, prec):
         g.close()
     for its, vm, va in out[1:]:
         assert np.array_equal(its, out[0][0]) and np.array_equal(vm, out[0][1]) and np.array_equal(va, out[0][2])
+
+
+# Grids of so many levels that the sweeps' steps take more shared memory than
+# set aside: the solve vector gives way, alone and in a pack (whose kernel has
+# less), instead of the whole run going to the one-case kernel.
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("n", [52000, 70000])
+def test_steps_of_many_levels_fit(n, prec):
+    case = gridgen.delaunay_raw(n, 7).scaled_network(1.0 / 512)
+    p = gbpf.PF_FP64 if prec == "fp64" else gbpf.PF_FP32
+    g = gbpf.Grid(case)
+    g.set_cases(1)
+    alone, packed = [], []
+    for tuning in (dict(tail=1, cluster=1), dict(), dict(tail=3, cluster=16)):
+        gbpf.pf_set_tuning(g.ctx, engine=gbpf.PF_ENGINE_BLOCK, **tuning)
+        alone.append(_run(g, n, 1, p, tol=1e-8, ir_tol=1e-3))
+    pk = gbpf.Pack([g])
+    for tuning in (dict(tail=1), dict()):
+        gbpf.pf_set_tuning(g.ctx, **tuning)
+        vm = torch.zeros(n, dtype=torch.float64, device="cuda")
+        va = torch.zeros_like(vm)
+        st, res = pk.run(gbpf.run_opts(gbpf.PF_FDPF, p, tol=1e-8, ir_tol=1e-3), vm, va)
+        packed.append((st, res, vm.cpu().numpy()[None], va.cpu().numpy()[None]))
+    pk.close()
+    g.close()
+    for st, res, vm, va in alone + packed:
+        assert st == gbpf.PF_OK and abs(int(res["iters"][0]) - int(alone[0][1]["iters"][0])) <= 1
+        # two mismatches within 1e-8, seen through the inverse Jacobian
+        assert np.abs(vm - alone[0][2]).max() <= 1e-5 and np.abs(va - alone[0][3]).max() <= 1e-5
+    if prec == "fp64" and n > 54000:  # half of the rows and the top do not fit shared memory
+        return
+    assert np.array_equal(alone[1][2], alone[2][2]) and np.array_equal(alone[1][3], alone[2][3])
+    # not the one-case kernels, whose bits tail 1 gives
+    assert not np.array_equal(alone[1][3], alone[0][3]) and not np.array_equal(packed[1][3], packed[0][3])
