@@ -274,7 +274,12 @@ pf_status pf_solve(pf_ctx *ctx, int32_t which, int32_t precision, int32_t transp
 /* Nodal P/Q mismatch (Section II.A) of the first ncase cases at the states
  * vm_dev/va_dev [ncase][nbus]: dp_dev/dq_dev [ncase][nbus] receive
  * Psp - P (non-slack, else 0) and Qsp - Q (PQ, else 0); maxmis_dev[ncase]
- * receives max |.|.  Uses each case's outage and load scale.  Asynchronous. */
+ * receives max |.|.  Uses each case's outage and load scale.  Errors are
+ * those of an FP64 evaluation or smaller: the nodal sums of ordinary buses
+ * run in fixed point, off by some 2^-59 of the row's sum of magnitudes,
+ * where FP64 loses as much; low voltages (below 9/16) and rows with few
+ * conductances or susceptances take FP64.  The same holds for pf_objective
+ * and pf_branch_flows.  Asynchronous. */
 pf_status pf_mismatch(pf_ctx *ctx, const double *vm_dev, const double *va_dev, double *dp_dev,
                       double *dq_dev, double *maxmis_dev, int32_t ncase, void *stream);
 
