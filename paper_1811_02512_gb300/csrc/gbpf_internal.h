@@ -338,8 +338,10 @@ struct DevNet {
     // (yst[i] = ysc[i], else kFxNoScale; rows64: some row is), and none of a
     // branch's six terms below 1/48 of their sum (q = kFxNoScale).  On a
     // lossless branch between angles of 1e-6 the flow was off by 3e-13 of
-    // itself, behind a tap of 1e-3 by 2e-14, 2e-16 in FP64.  The iteration,
-    // which ends at a tolerance on the absolute mismatch, takes ysc.
+    // itself, behind a tap of 1e-3 by 2e-14, 2e-16 in FP64.  (10,000 buses x 256
+    // without any resistance: mismatch 350 us and flows 1,115, 160 and 234 in
+    // fixed point.)  The iteration, which ends at a tolerance on the absolute
+    // mismatch, takes ysc.
     int *ysc = nullptr, *yesc = nullptr, *yst = nullptr;
     int rows64 = 0;
     int4 *Yx = nullptr, *bryx = nullptr;
